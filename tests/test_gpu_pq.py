@@ -153,3 +153,76 @@ def test_pipeline_with_pq_latents_keeps_the_bounds(aq):
     qf, qx = f @ phi.T * vol, xx @ phi.T * vol
     sk = np.abs(xx) @ np.abs(phi).T * vol
     assert np.max(np.abs(qf - qx) / sk) <= 1e-10
+
+
+@pytest.mark.parametrize("k", [2, 3, 16, 33, 256])
+def test_assignment_any_table(aq, k):
+    """The bisection gives the index of the full search (and the oracle's) for
+    every table a caller may pass: ascending, with equal or adjacent-float or
+    descending neighbours, with infinities and NaN; at centroids, midpoints,
+    their neighbouring floats, and values far outside the table."""
+    rng = np.random.default_rng(k)
+    L = 8
+    t = np.sort(rng.standard_normal((L, k)).astype(np.float32), axis=1)
+    t[1, k // 2] = t[1, k // 2 - 1]
+    t[2, k // 2] = np.nextafter(t[2, k // 2 - 1], np.float32(9))
+    t[3] = t[3][::-1]
+    t[4] = (1e7 + np.arange(k)).astype(np.float32)
+    t[5, -1] = np.inf
+    t[6, 0] = np.nan
+    t[7] = (t[7] * np.float32(1e-42)).astype(np.float32)
+    with np.errstate(invalid="ignore", over="ignore"):
+        mid = (t[:, :-1] + t[:, 1:]) / np.float32(2)
+        cols = [t, mid, np.nextafter(mid, np.float32(9)), np.nextafter(mid, np.float32(-9)),
+                np.nextafter(t, np.float32(9)), rng.standard_normal((L, 64)).astype(np.float32),
+                np.tile(np.float32([0, -0.0, 1e30, -1e30, 3e38, np.inf, -np.inf, np.nan, 1e-45,
+                                    16777216, 0.4]), (L, 1)),
+                t[:, :1] - np.float32(4194304) * (t[:, 1:2] - t[:, :1]) *
+                np.float32([[0.25, 0.5, 0.75, 1, 2]])]
+        z = np.ascontiguousarray(np.concatenate(cols, axis=1).T.astype(np.float32))
+        # the full search starts from centroid 0, whose NaN distance nothing beats
+        ref = np.zeros(z.shape, np.uint8)
+        best = np.abs(z - t[:, 0])
+        for j in range(1, k):
+            d = np.abs(z - t[:, j])
+            ref[d < best] = j
+            best = np.where(d < best, d, best)
+        fin = ~np.isnan(t).any(axis=1)
+        np.testing.assert_array_equal(ref[:, fin], opq.assign(z, t)[:, fin])
+    codes, _ = aq.pq_encode(torch.as_tensor(z, device=DEV), torch.as_tensor(t[None], device=DEV))
+    np.testing.assert_array_equal(codes.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("n,L", [(1, 32), (7, 16), (4097, 32), (3001, 5)])
+def test_one_iteration_wide_magnitudes(aq, n, L):
+    """Means of columns whose values span 40 binades, subnormals among them
+    (shifts either side of the fixed point's last place), at row counts around
+    the unrolled loads of a block."""
+    rng = np.random.default_rng(n)
+    z = (rng.standard_normal((n, L)) * 2.0 ** rng.uniform(-30, 10, (n, L))).astype(np.float32)
+    z[:, L // 2] *= np.float32(2.0 ** -130)
+    t = aq.pq_train(torch.as_tensor(z, device=DEV), k=16, iters=1).cpu().numpy()[0]
+    ref = opq.train(z, 16, 1)
+    assert np.all(np.abs(t - ref) <= table_tol(z, ref))
+
+
+@pytest.mark.parametrize("n,L,G,k,kind", [
+    (20000, 32, 1, 16, "normal"), (20000, 5, 2, 16, "normal"), (150000, 16, 2, 16, "normal"), (70000, 8, 1, 16, "patterns"), (3000, 16, 5, 16, "normal"),
+    (70000, 8, 1, 256, "normal"), (200000, 3, 1, 16, "patterns"), (5000, 8, 1, 2, "offset")])
+def test_bf16_counts_equal_values(aq, n, L, G, k, kind):
+    """bfloat16 latents (counted by value) and the same values as float32
+    (summed one by one) give the same tables bit for bit: few and very many
+    distinct values, non-finite patterns, ragged groups, rows that are not
+    multiples of eight elements, an unaligned first row."""
+    rng = np.random.default_rng(n + L)
+    if kind == "patterns":
+        z = torch.as_tensor(rng.integers(0, 65536, (n + 1, L)).astype(np.uint16).view(np.int16),
+                            device=DEV).view(torch.bfloat16)
+    else:
+        z = torch.as_tensor(latents(n + 1, L, n), device=DEV).to(torch.bfloat16)
+    z = z[1:] if kind == "offset" else z[:n].contiguous()
+    off = np.sort(np.concatenate([[0, n], rng.integers(0, n, G - 1)])).astype(np.int64)
+    goff = torch.as_tensor(off, device=DEV) if G > 1 else None
+    a = aq.pq_train(z, k=k, iters=6, group_offsets=goff, G=G)
+    b = aq.pq_train(z.float(), k=k, iters=6, group_offsets=goff, G=G)
+    np.testing.assert_array_equal(a.cpu().numpy().view(np.int32), b.cpu().numpy().view(np.int32))
