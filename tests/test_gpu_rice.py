@@ -105,3 +105,25 @@ def test_damaged_streams_stay_in_bounds(aq):
     # histograms whose stream and offsets are intact still decode exactly
     ok = [b for b in range(64) if b not in (4, 5, 8, 9, 19, 20)]
     np.testing.assert_array_equal(d2.cpu().numpy()[ok], q[ok])
+
+
+@pytest.mark.parametrize("P,n,shift", [(992, 9, 0), (993, 9, 1), (1087, 5, 0), (1088, 6, 1),
+                                       (1221, 40, 1), (1521, 1, 1), (1521, 7, 0), (1536, 5, 1),
+                                       (64, 33, 1)])
+def test_streams_any_alignment(aq, P, n, shift):
+    """Rows around the run lengths of the packer, on even and odd 2-byte
+    boundaries, alone or next to others; every width of code from all-zero to
+    all-escaped, so that both staged and unstaged streams and every k occur."""
+    q = np.concatenate([mixed_codes(max(n, 4), P, P + n)])[:n]
+    rng = np.random.default_rng(P)
+    for r in range(4, n, 5):  # a few wide codes among zeros: capped prefixes at the best k
+        q[r] = np.where(rng.random(P) < 0.02, rng.integers(-32766, 32767, P), rng.integers(0, 2, P))
+    flat = torch.full((n * P + 2,), 12345, dtype=torch.int16, device=DEV)
+    flat[shift:shift + n * P] = torch.as_tensor(q.reshape(-1), device=DEV)
+    rs = aq.rice_encode(flat[shift:shift + n * P].view(n, P))
+    ks, nb, off, words = orice.encode(q)
+    np.testing.assert_array_equal(rs.kparam.cpu().numpy(), ks)
+    np.testing.assert_array_equal(rs.nbits.cpu().numpy().astype(np.uint32), nb)
+    np.testing.assert_array_equal(rs.offsets.cpu().numpy(), off)
+    np.testing.assert_array_equal(rs.words.cpu().numpy().view(np.uint32), words)
+    np.testing.assert_array_equal(aq.rice_decode(rs, P).cpu().numpy(), q)
