@@ -163,8 +163,8 @@ struct FusedArgs {
 };
 
 int launch_fused_fp64(const FusedArgs& a, cudaStream_t s);
-int launch_fused_fp64_list(const FusedArgs& a, const int* list, const int* count,
-                           cudaStream_t s);
+// the listed histograms (completed entries are overwritten)
+int launch_fused_fp64_list(const FusedArgs& a, int* list, int* count, cudaStream_t s);
 // fast kernel + FP64 kernel over its deferred list; fb_list [n] and fb_count
 // are scratch in device memory
 int launch_fused_fast(const FusedArgs& a, cudaStream_t s, int warps_per_sm = 0);

@@ -503,3 +503,71 @@ def test_bin_width_at_binade_carries_matches_oracle(aq, grids, tau):
     check_batch(aq, og, x, xh, tau, aq.KERNEL_FAST, n_expect_conv=0.9)
     dl = np.array([oracle.delta(tau * s, 0.5) for s in svals])
     assert len(np.unique(np.log2(dl[:len(carry)]))) > 1  # several binades
+
+
+@pytest.mark.parametrize("n,grid,cap", [(1, (39, 39), 4000), (77, (39, 39), 4000),
+                                        (320, (39, 39), 100000), (90, (37, 33), 50),
+                                        (40, (64, 24), 4000), (25, (2, 5), 100),
+                                        (30, (1, 64), 100)])
+def test_cluster_form_equals_warp_form(aq, n, grid, cap):
+    """A small batch (a cluster of blocks per histogram) gives what the same
+    rows give inside a large one (a warp per histogram): codes, scales,
+    statuses, step counts and outliers exactly, multipliers and corrected
+    values to the rounding of the sums' order (1e-9 of their size, the
+    multipliers' own tolerance being 1e-12 of the moments)."""
+    npar, nperp = grid
+    vpar, vperp, vol = synth.grid_arrays(*grid) if npar > 1 else (np.zeros(1),
+                                                                  np.linspace(0, 4, nperp), 0.1)
+    g = aq.Grid(vpar, vperp, vol)
+    P = npar * nperp
+    rng = np.random.default_rng(n)
+    if npar > 1:
+        x = synth.histograms(n, synth.config_seed(9), grid=grid)
+    else:
+        x = rng.random((n, P))
+    xh = synth.stand_in_xhat(x, 5)
+    for r in range(1, n, 9):
+        k = (r // 9) % 7
+        c = rng.integers(0, P)
+        if k == 0:
+            x[r] = 0.0
+        elif k == 1:
+            x[r, c] = np.nan
+        elif k == 2:
+            x[r, c] = -1e-3
+        elif k == 3:
+            xh[r, c] = np.inf
+        elif k == 4:
+            xh[r, :P] += np.float32(3e4 * 1e-4 * x[r].max())
+        elif k == 5:
+            xh[r, : P // 2] = np.float32(1e9)
+        else:  # every point a little off: the bound fails at both levels
+            xh[r, :P] = (x[r] + 0.49e-4 * x[r].max()).astype(np.float32)
+    p = aq.params_default(tau=1e-4, kernel=aq.KERNEL_FP64)
+    reps = 1100 // n + 1
+    small = aq.quantize_correct(g, dev(x), dev(xh), p, outlier_capacity=cap, want_f=True)
+    big = aq.quantize_correct(g, dev(np.tile(x, (reps, 1))), dev(np.tile(xh, (reps, 1))), p,
+                              outlier_capacity=reps * cap, want_f=True)
+    torch.cuda.synchronize()
+    get = lambda t: t[:n].cpu().numpy()  # noqa: E731
+    over = oracle.OUTLIER_OVERFLOW if hasattr(oracle, "OUTLIER_OVERFLOW") else 0x200
+    assert np.array_equal(get(small.codes), get(big.codes))
+    assert np.array_equal(get(small.scale), get(big.scale), equal_nan=True)
+    assert np.array_equal(get(small.iters), get(big.iters))
+    assert np.array_equal(get(small.status) & ~np.uint16(over), get(big.status) & ~np.uint16(over))
+    assert np.allclose(get(small.lam), get(big.lam), rtol=1e-9, atol=1e-12)
+    fs, fb = get(small.f), get(big.f)
+    ok = np.isfinite(x)
+    scale = np.where(ok, np.abs(x), 0).max(axis=1, keepdims=True)
+    assert np.array_equal(np.isfinite(fs), np.isfinite(fb))
+    assert np.all(np.abs(fs - fb)[ok] <= (1e-9 * np.broadcast_to(scale, x.shape))[ok])
+    # outliers: the same set of rows' entries, in point order within a row
+    m, total = int(small.count.item()), int(big.count.item())
+    assert total == reps * m
+    if m <= cap:
+        i1, v1 = small.index[:m].cpu().numpy(), small.value[:m].cpu().numpy()
+        i2, v2 = big.index[:total].cpu().numpy(), big.value[:total].cpu().numpy()
+        keep = i2 < n * P
+        o1, o2 = np.argsort(i1), np.argsort(i2[keep])
+        assert np.array_equal(i1[o1], i2[keep][o2])
+        assert np.array_equal(v1[o1], v2[keep][o2], equal_nan=True)
