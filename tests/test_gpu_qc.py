@@ -571,3 +571,45 @@ def test_cluster_form_equals_warp_form(aq, n, grid, cap):
         o1, o2 = np.argsort(i1), np.argsort(i2[keep])
         assert np.array_equal(i1[o1], i2[keep][o2])
         assert np.array_equal(v1[o1], v2[keep][o2], equal_nan=True)
+
+
+@pytest.mark.parametrize("tau", [1e-4, 0.3, 1e-30, 4e-300])
+def test_decompressed_values_are_the_fp64_form(aq, tau):
+    """f = fl(fl(fl(xhat + q Delta) a) b) bit for bit, for codes and decoded
+    values in every relation to each other (equal and opposite, far apart,
+    subnormal, zero of either sign, non-finite, zero-level codes); a is read
+    off the point whose x' is 1, with lambda_0 alone so that b = 1."""
+    P, n = 1521, 24
+    rng = np.random.default_rng(3)
+    mu = (rng.standard_normal(P) * 2.0 ** rng.uniform(-60, 20, P)).astype(np.float32)
+    mu[:40] *= np.float32(2.0 ** -100)
+    dl = 2.0 ** np.floor(np.log2(tau))
+    q = np.rint(rng.standard_normal((n, P)) * 10.0 ** rng.uniform(0, 4.4, (n, 1))).astype(np.int16)
+    q[:, 5::50] = oracle.ZERO_CODE if hasattr(oracle, "ZERO_CODE") else -32767
+    q[:, 7::30] = 0
+    if 1e-30 <= tau < 1:  # decoded values on the code lattice: exact cancellation
+        mu[9::20] = (-q[0, 9::20].astype(np.float64) * dl).astype(np.float32)
+    mu[100:106] = [0.0, -0.0, np.inf, np.nan, -np.inf, 1e-45]
+    mu[0], q[:, 0] = 1.0, 0
+    lam = np.zeros((n, 4))
+    lam[1:, 0] = rng.standard_normal(n - 1) * 10.0 ** rng.uniform(-12, 0.5, n - 1)
+    lam[n - 1, 0] = 40.0
+    m = aq.Model(P, 32, 8)
+    z = lambda *s: np.zeros(s)  # noqa: E731
+    m.set_group(0, dict(W1=z(P, 32), b1=z(32), W2=z(32, 8), b2=z(8), b3=z(32), b4=z(P),
+                        mu=mu.astype(np.float64), sigma=np.ones(P)))
+    c = aq.Compressed(n, P, 8, torch.float32, DEV, 16)
+    c.latent.zero_()
+    c.scale.fill_(1.0)
+    c.codes.copy_(dev(q))
+    c.lam.copy_(dev(lam))
+    c.status.copy_(dev(np.ones(n, np.uint16)))
+    f = aq.decompress_batch(m, aq_grid(aq), c, aq.params_default(tau=tau)).cpu().numpy()
+    xhat = aq.ae_decode(m, c.latent, c.scale)[:, :P].cpu().numpy()
+    a = f[:, :1]
+    assert np.all(np.abs(a - np.exp(-lam[:, :1])) <= np.spacing(np.exp(-lam[:, :1])))
+    with np.errstate(invalid="ignore", over="ignore"):
+        xp = np.where(q == -32767, 0.0, xhat.astype(np.float64) + q.astype(np.float64) * dl)
+        want = xp * a
+    np.testing.assert_array_equal(f, want)
+    assert np.array_equal(np.signbit(f), np.signbit(want)) or np.isnan(want).any()
