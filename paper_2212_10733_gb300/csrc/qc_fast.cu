@@ -255,54 +255,80 @@ __device__ __noinline__ PointQ quant_point_hard(double x, float xh, double dl) {
   return o;
 }
 
+// Logical right shift of 64 bits by any unsigned amount (0 from 64 on).
+__device__ __forceinline__ unsigned long long shr64(unsigned long long v, unsigned n) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+
+__device__ __forceinline__ unsigned long long pack64(unsigned lo, unsigned hi) {
+  return ((unsigned long long)hi << 32) | lo;
+}
+
+// X = floor(x / u) for x >= 0 (+0 and subnormals give 0, and so does -0)
+__device__ __forceinline__ unsigned long long x_units(unsigned long long ux, const QConst& c) {
+  const unsigned xh = (unsigned)(ux >> 32), xl = (unsigned)ux;
+  // mantissa with its implicit bit at bits 10..62; where there is no implicit
+  // bit the shift below passes 63
+  const unsigned mh = (__funnelshift_l(xl, xh, 10) & 0x3FFFFFFFu) | 0x40000000u;
+  return shr64(pack64(xl << 10, mh), (unsigned)(c.cx - (int)(xh >> 20)));
+}
+
 // Quantizer decision for one point (x finite, x >= 0), exact where it is
 // not flagged.  With u = Delta 2^-38, X = floor(x / u) and Xh = trunc(xhat / u)
 // come from the bit patterns; the exact scaled difference (x - xhat) / u is
 // D + e with D = X - Xh and e in (-1, 2).  With t = D + 2^37, q = floor(t / 2^38)
 // is the round-half-even index unless t's fraction is within two units of a
-// multiple of 2^38 (a tie or an uncertain rounding): that point is flagged.
-// rho = D - q 2^38 is the residual (x - xhat - q Delta) / u within the same
-// (-1, 2) units; the zero level wins iff |x - xhat - q Delta| > x, decided on
-// |rho| - X unless within three units (flagged).  Escapes (|q| > 32766 or a
-// non-finite or huge xhat) are flagged too.  A flagged point's outputs here
-// are zero; the caller completes it with the exact FP64 routine.
+// multiple of 2^38 (a tie or an uncertain rounding): that point is flagged (on
+// the upper 31 bits of the fraction, a band of 128 units).  rho = D - q 2^38 is
+// the residual (x - xhat - q Delta) / u within the same (-1, 2) units.  The zero
+// level wins iff x' = xhat + q Delta < 0, which the rounded xpf decides exactly
+// (a sum of two multiples of 2^-149 that is not zero does not round to it), or
+// x' > 2x, which is decided on X + rho unless within three units (flagged).
+// Escapes (|q| > 32766) are flagged too; |xhat| from 2^23 Delta up, infinite or
+// NaN, is at least 2^61 units here, so that its q is one.  x' >= 0 gives
+// X - rho >= 0.  The caller completes a flagged point with the exact FP64
+// routine.
+// Bound: the integer (ALU) pipe, about 110 instructions a point with the moment
+// sums.  On 32-bit words where one decides, shifts without clamps, no select
+// for the residual: 1,048,576 histograms in compress 23.17 -> 21.70 ms, with the
+// row maximum, the fold and the pass's reductions below.
 struct PointF {
-  int code;       // q, or AEQC_CODE_ZERO (0 when flagged)
-  long long xpw;  // x' / u within one unit (0 when flagged or at the zero level)
-  long long rho;  // (x - x') / u within two units (0 when flagged)
-  float xpf;      // x' as a float (0 when flagged or at the zero level)
+  int code;                // q, or AEQC_CODE_ZERO (any value when flagged)
+  unsigned long long X;    // x / u, truncated
+  unsigned long long xpw;  // x' / u within one unit (0 when flagged or at the zero level)
+  int r31;                 // (x - x') / Delta 2^31, rounded down
+  float xpf;               // x' as a float (0 when flagged or at the zero level)
   bool hard;
 };
+// marks a flagged point in the residual array: residuals lie within +-2^14
+constexpr int RHO_HARD = -32768;
 
 __device__ __forceinline__ PointF quant_point_fast(double x, float xh, const QConst& c) {
-  const unsigned long long ux = (unsigned long long)__double_as_longlong(x);
-  const int E = (int)(ux >> 52);  // x >= 0: no sign bit
-  // mantissa with its implicit bit at bits 10..62; a subnormal x gives X = 0
-  const unsigned long long M10 =
-      ((ux & 0xFFFFFFFFFFFFFull) | ((unsigned long long)(E != 0) << 52)) << 10;
-  const long long X = (long long)(M10 >> min(c.cx - E, 63));
-  const unsigned v = __float_as_uint(xh);
-  const int Eh = (v >> 23) & 0xff;
-  const bool esc_h = Eh >= c.thr;  // |q| > 32766 for sure, or a non-finite xhat
-  const unsigned long long m40 = (unsigned long long)((v & 0x7fffffu) | (Eh ? 0x800000u : 0u))
-                                 << 40;
-  const long long mag = (long long)(m40 >> min(max(c.ch - (Eh ? Eh : 1), 0), 63));
-  const long long D = X - ((v >> 31) ? -mag : mag);
-  const long long t = D + (1ll << (QF - 1));
-  const int q = (int)(t >> QF);
-  const bool band = ((t + 2) & ((1ll << QF) - 1)) < 4;
-  const long long rho = D - ((long long)q << QF);
-  const long long uz = (rho < 0 ? -rho : rho) - X;  // |r| - x in units
-  const bool zero = uz > 3;
-  const bool band2 = (unsigned long long)(uz + 3) <= 6ull;
   PointF o;
-  o.hard = band || band2 || esc_h || q > AEQC_CODE_MAX || q < -AEQC_CODE_MAX;
-  const bool keep = !o.hard && !zero;
-  o.code = o.hard ? 0 : (zero ? AEQC_CODE_ZERO : q);
-  o.xpw = keep ? X - rho : 0ll;
-  o.rho = o.hard ? 0ll : (zero ? X : rho);
+  o.X = x_units((unsigned long long)__double_as_longlong(x), c);
+  const unsigned v = __float_as_uint(xh);
+  const int sh = max(c.ch - (int)((v << 1) >> 24), 1);
+  const unsigned long long sm = (unsigned long long)(long long)((int)v >> 31);
+  const unsigned long long D =
+      o.X - (shr64(pack64(0u, (v << 8) | 0x80000000u), (unsigned)sh) ^ sm) + sm;
+  const int Dh = (int)(D >> 32);
+  const int q = (Dh + (1 << (QF - 33))) >> (QF - 32);
+  const int rh = Dh - q * (1 << (QF - 32));
+  const unsigned long long rho = pack64((unsigned)D, (unsigned)rh);
+  const int r31 = (int)__funnelshift_r((unsigned)D, (unsigned)rh, QF - 31);
+  const unsigned long long b3 = o.X + rho + 3ull;
   // |q| < 2^22 wherever the value is kept
-  o.xpf = keep ? fmaf(small_int_to_float(q), c.dl_f, xh) : 0.f;
+  const float xpf = fmaf(small_int_to_float(q), c.dl_f, xh);
+  o.hard = (unsigned)(r31 + 0x3FFFFFFF) >= 0x7FFFFFFEu ||
+           (unsigned)(q + AEQC_CODE_MAX) > 2u * AEQC_CODE_MAX || b3 <= 6ull;
+  const bool zero = xpf < 0.f || (long long)b3 < 0;
+  const bool keep = !o.hard && !zero;
+  o.code = zero ? AEQC_CODE_ZERO : q;
+  o.xpw = keep ? o.X - rho : 0ull;
+  o.r31 = zero ? (int)(unsigned)(o.X >> (QF - 31)) : r31;
+  o.xpf = keep ? xpf : 0.f;
   return o;
 }
 
@@ -384,47 +410,57 @@ __device__ __forceinline__ void lane_segments(const FastGridK& fg, int n_par, in
   }
 }
 
-// Column sums of one segment: X' j^(2q) (split at bit 31), rho j^(2q)
+// Column sums of one segment: X' j^(2q) (split at bit 32), X j^(2q) modulo 2^64
 // (q = 0, 1) and x' (float).
 struct ColSums {
-  long long b[3], a[3], u[2];
+  unsigned long long b[3], a[3], u[2];
   float xs;
 };
 
 // a + b c for unsigned 32-bit b, c (one wide multiply-add)
-__device__ __forceinline__ long long mad_wide(long long a, unsigned b, unsigned c) {
-  return (long long)((unsigned long long)a + (unsigned long long)b * (unsigned long long)c);
+__device__ __forceinline__ unsigned long long mad_wide(unsigned long long a, unsigned b,
+                                                       unsigned c) {
+  return a + (unsigned long long)b * (unsigned long long)c;
 }
 
-__device__ __forceinline__ void colsum_add(ColSums& cs, long long xpw, long long rho, float xpf,
-                                           unsigned j2, unsigned j4) {
-  // x' >= 0 here, below 2^60 units: two unsigned 32-bit parts (31 + 29 bits)
-  const unsigned xl = (unsigned)xpw & 0x7FFFFFFFu, xu = (unsigned)(xpw >> 31);
+__device__ __forceinline__ void colsum_add_xp(ColSums& cs, unsigned long long xpw, float xpf,
+                                              unsigned j2, unsigned j4) {
+  // x' >= 0, below 2^60 units (and the grid's sum of every weight below 2^31,
+  // host check): two unsigned parts
+  const unsigned xl = (unsigned)xpw, xu = (unsigned)(xpw >> 32);
   cs.b[0] += xl;
   cs.b[1] = mad_wide(cs.b[1], xl, j2);
   cs.b[2] = mad_wide(cs.b[2], xl, j4);
   cs.a[0] += xu;
   cs.a[1] = mad_wide(cs.a[1], xu, j2);
   cs.a[2] = mad_wide(cs.a[2], xu, j4);
-  // |rho| <= 2^37 and the grid's sum of j^2 is below 2^25 (host check):
-  // every total stays below 2^62.  rho j2 from rho's two words, modulo 2^64
-  // (two's complement: the exact product).
-  cs.u[0] += rho;
-  cs.u[1] = mad_wide(cs.u[1] + (long long)((unsigned long long)((unsigned)(rho >> 32) * j2) << 32),
-                     (unsigned)rho, j2);
   cs.xs += xpf;
+}
+
+// The residual sums are those of X less those of X': only their difference has
+// to fit in 64 bits, and a point at the zero level needs no case of its own.
+__device__ __forceinline__ void colsum_add_x(ColSums& cs, unsigned long long X, unsigned j2) {
+  cs.u[0] += X;
+  cs.u[1] = mad_wide(cs.u[1], (unsigned)X, j2) +
+            ((unsigned long long)((unsigned)(X >> 32) * j2) << 32);
+}
+
+// sum rho j^(2q) of a segment (|rho| <= 2^37 and the grid's sum of j^2 below
+// 2^25, host check: below 2^62)
+__device__ __forceinline__ long long rho_sum(const ColSums& cs, int q) {
+  return (long long)(cs.u[q] - cs.b[q] - (cs.a[q] << 32));
 }
 
 // Quantize one segment (column sg.c, rows [j0, j1)): codes to cb (global), x'
 // and the residual (in Delta 2^-15) to shared memory, column sums to cs.  One
-// straight-line body per point; the flagged points (a bit per row of the
-// segment, at most 64 rows) are completed after the walk.
+// straight-line body per point; the flagged points are marked in the residual
+// array and completed after the walk.
 __device__ __forceinline__ void quant_segment(const Seg& sg, int n_par, const double* xb,
                                               const float* xhb, const QConst& c, FastWS& w,
                                               int16_t* cb, ColSums& cs, int& esc,
                                               int& nonzero) {
   cs = ColSums{{0, 0, 0}, {0, 0, 0}, {0, 0}, 0.f};
-  unsigned long long flagged = 0;
+  int hard = 0;
   int nz = 0;
   int p = sg.j0 * n_par + sg.c;
   // loads issued two points ahead of the work
@@ -446,27 +482,38 @@ __device__ __forceinline__ void quant_segment(const Seg& sg, int n_par, const do
     const PointF o = quant_point_fast(x, xh, c);
     cb[p] = (int16_t)o.code;
     w.xp[p] = o.xpf;
-    w.rho[p] = (int16_t)((o.rho + (1ll << 22)) >> 23);
+    // the residual to Delta 2^-15, rounded
+    w.rho[p] = (int16_t)(o.hard ? RHO_HARD : (o.r31 + (1 << 15)) >> 16);
     nz |= o.code;
-    if (o.hard) flagged |= 1ull << (j - sg.j0);
-    colsum_add(cs, o.xpw, o.rho, o.xpf, j2, j2 * j2);
+    hard = o.hard ? 1 : hard;
+    colsum_add_xp(cs, o.xpw, o.xpf, j2, j2 * j2);
+    colsum_add_x(cs, o.X, j2);
     j2 += 2 * j + 1;  // (j + 1)^2
   }
-  nonzero |= nz;
   // the flagged points: the exact FP64 routine (out of line), outputs stored
-  // and moments added
-  while (flagged) {
-    const int j = sg.j0 + __ffsll((long long)flagged) - 1;
-    flagged &= flagged - 1;
-    const int pf = j * n_par + sg.c;
-    const PointQ o = quant_point_hard(__ldg(xb + pf), __ldg(xhb + pf), c.dl);
-    cb[pf] = (int16_t)o.code;
-    w.xp[pf] = o.xpf;
-    w.rho[pf] = (int16_t)((o.rho + (1ll << 22)) >> 23);
-    esc |= o.code == AEQC_CODE_ESCAPE;
-    nonzero |= o.code != 0;
-    colsum_add(cs, o.xpw, o.rho, o.xpf, (unsigned)(j * j), (unsigned)(j * j * j * j));
+  // and moments added (X is in the sums already)
+  if (hard) {
+    nz = 0;
+    p = sg.j0 * n_par + sg.c;
+#pragma unroll 1
+    for (int j = sg.j0; j < sg.j1; ++j, p += n_par) {
+      if (w.rho[p] == RHO_HARD) {
+        const double x = __ldg(xb + p);
+        const PointQ o = quant_point_hard(x, __ldg(xhb + p), c.dl);
+        cb[p] = (int16_t)o.code;
+        w.xp[p] = o.xpf;
+        w.rho[p] = (int16_t)((o.rho + (1ll << 22)) >> 23);
+        esc |= o.code == AEQC_CODE_ESCAPE;
+        const unsigned jj = (unsigned)(j * j);
+        colsum_add_xp(cs, (unsigned long long)o.xpw, o.xpf, jj, jj * jj);
+        // the routine's own rounding of the residual
+        const unsigned long long X = x_units((unsigned long long)__double_as_longlong(x), c);
+        colsum_add_x(cs, (unsigned long long)(o.rho + o.xpw) - X, jj);
+      }
+      nz |= cb[p];
+    }
   }
+  nonzero |= nz;
 }
 
 // Quantize the histogram (row xb, decoded row xhb): codes to cb (global),
@@ -482,28 +529,36 @@ __device__ void phase_a(const GridK& g, const FastGridK& fg, const double* xb,
   quant_segment(sg2, g.n_par, xb, xhb, c, w, cb, c2, esc, nonzero);
   // fold with the powers of i - i_c: U_q over weights 1, ic, ic^2, j^2 and T
   // over (ic^r j^(2q)) in the order T00 T10 T20 T30 T40 T01 T11 T21 T02, the
-  // latter as Tb + 2^31 Ta
+  // latter as Tb + 2^32 Ta (totals below 2^63)
   long long U[4], Tb[9], Ta[9];
   {
-    const long long i1 = sg1.c - fg.i_c, i2 = sg2.c - fg.i_c;
-    const long long p1[5] = {1, i1, i1 * i1, i1 * i1 * i1, i1 * i1 * i1 * i1};
-    const long long p2[5] = {1, i2, i2 * i2, i2 * i2 * i2, i2 * i2 * i2 * i2};
+    // v ic^r: the even powers as unsigned words, the odd ones with a sign
+    const int i1 = sg1.c - fg.i_c, i2 = sg2.c - fg.i_c;
+    auto times = [](unsigned long long v, int i, int r) -> unsigned long long {
+      const unsigned e = (unsigned)(i * i);
+      if (r == 0) return v;
+      if (r == 2) return v * e;
+      if (r == 4) return v * (e * e);
+      return v * (unsigned long long)(long long)(r == 1 ? i : i * (int)e);
+    };
     const int rq[9][2] = {{0, 0}, {1, 0}, {2, 0}, {3, 0}, {4, 0}, {0, 1}, {1, 1}, {2, 1}, {0, 2}};
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
       const int r = rq[k][0], q = rq[k][1];
-      Tb[k] = c1.b[q] * p1[r] + c2.b[q] * p2[r];
-      Ta[k] = c1.a[q] * p1[r] + c2.a[q] * p2[r];
+      Tb[k] = (long long)(times(c1.b[q], i1, r) + times(c2.b[q], i2, r));
+      Ta[k] = (long long)(times(c1.a[q], i1, r) + times(c2.a[q], i2, r));
     }
+    const unsigned long long u1 = (unsigned long long)rho_sum(c1, 0),
+                             u2 = (unsigned long long)rho_sum(c2, 0);
 #pragma unroll
-    for (int r = 0; r < 3; ++r) U[r] = c1.u[0] * p1[r] + c2.u[0] * p2[r];
-    U[3] = c1.u[1] + c2.u[1];
+    for (int r = 0; r < 3; ++r) U[r] = (long long)(times(u1, i1, r) + times(u2, i2, r));
+    U[3] = rho_sum(c1, 1) + rho_sum(c2, 1);
   }
   const float b_f = fg.b_f, c0_f = fg.c0_f;
   float s1 = c1.xs * fabsf(fmaf(b_f, small_int_to_float(sg1.c - fg.i_c), c0_f)) +
              c2.xs * fabsf(fmaf(b_f, small_int_to_float(sg2.c - fg.i_c), c0_f));
   __syncwarp();
-  // exact warp totals (the host bounds them below 2^62), scattered over the
+  // exact warp totals (the host bounds them below 2^63), scattered over the
   // lanes: lane k holds total k of (U0..U3, Tb0..Tb8, Ta0..Ta8); each lane
   // converts one total to double-float
   long long v[32];
@@ -513,7 +568,7 @@ __device__ void phase_a(const GridK& g, const FastGridK& fg, const double* xb,
   df mine = df_from_ll(reduce_scatter32(v, lane));
   {
     const df ta = {__shfl_down_sync(FULL, mine.hi, 9), __shfl_down_sync(FULL, mine.lo, 9)};
-    if (lane >= 4 && lane < 13) mine = df_add(df_ldexp(ta, 31), mine);  // T = Tb + 2^31 Ta
+    if (lane >= 4 && lane < 13) mine = df_add(df_ldexp(ta, 32), mine);  // T = Tb + 2^32 Ta
   }
   float S1 = s1;
 #pragma unroll
@@ -618,19 +673,6 @@ __device__ void pass_warp(const GridK& g, const FastGridK& fg, const FastWS& w,
   // order m00 m10 m20 m30 m40 m01 m11 m21 m02 (w^q as j^(2q), d2^q later)
   float jz[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   const float cq = c.dl_f * 3.0517578125e-05f, dq = -12582912.f * cq;  // Delta 2^-15
-  // x' h(t), x' h'(t) and the check value of one point (the largest check
-  // value decides the check after the walk); h'(t) = 1 - e^-t = t - h(t)
-  auto point = [&](int p, float t, float& z) -> float {
-    const float xp = w.xp[p];
-    const float h =
-        t * t * fmaf(-t, fmaf(-t, fmaf(-t, 1.f / 120.f, 1.f / 24.f), 1.f / 6.f), 0.5f);
-    // Delta rho from its 2^-15 fixed point: exact, see small_int_to_float
-    const float drho = fmaf(__int_as_float(0x4B400000 + (int)w.rho[p]), cq, dq);
-    const float hmt = h - t;
-    errmax = fmaxf(errmax, fabsf(fmaf(xp, hmt, -drho)));
-    z = -xp * hmt;
-    return xp * h;
-  };
   Seg sg[2];
   lane_segments(fg, g.n_par, g.n_perp, lane, sg[0], sg[1]);
 #pragma unroll 1
@@ -645,26 +687,38 @@ __device__ void pass_warp(const GridK& g, const FastGridK& fg, const FastWS& w,
     const float ah = A.hi, al = A.lo;
     df s0 = {0.f, 0.f}, s3 = {0.f, 0.f};
     float z0 = 0.f, z1 = 0.f, z2 = 0.f;  // sums of z, z j^2, z j^4
-    float jf = small_int_to_float(sgm.j0), j2f = jf * jf;
+    const float j0f = small_int_to_float(sgm.j0);
     // |t| is largest at an end of the segment (t is monotone in j^2): a bound
     // over every point of the segment, x' = 0 included
     if (sgm.j1 > sgm.j0) {
       const float jl = small_int_to_float(sgm.j1 - 1);
-      tmax = fmaxf(tmax, fmaxf(fabsf(fmaf(tc.h[2], j2f, ah)), fabsf(fmaf(tc.h[2], jl * jl, ah))));
+      tmax = fmaxf(tmax, fmaxf(fabsf(fmaf(tc.h[2], j0f * j0f, ah)),
+                               fabsf(fmaf(tc.h[2], jl * jl, ah))));
     }
+    // x' h(t), x' h'(t) (h'(t) = 1 - e^-t = t - h(t)) and the check value of a
+    // point (the largest check value decides the check after the walk).  Every
+    // rounding is written out: the step counts must not depend on contraction.
+    float jf = j0f, j2f = j0f * j0f;
     int p = sgm.j0 * g.n_par + sgm.c;
     for (int j = sgm.j0; j < sgm.j1; ++j, p += g.n_par) {
-      const float t = fmaf(tc.h[2], j2f, ah) + fmaf(tc.l[2], j2f, al);
-      float z;
-      const float y = point(p, t, z);
-      z0 += z;
+      const float t = __fadd_rn(fmaf(tc.h[2], j2f, ah), fmaf(tc.l[2], j2f, al));
+      const float xp = w.xp[p];
+      const float h = __fmul_rn(
+          __fmul_rn(t, t),
+          fmaf(-t, fmaf(-t, fmaf(-t, 1.f / 120.f, 1.f / 24.f), 1.f / 6.f), 0.5f));
+      // Delta rho from its 2^-15 fixed point: exact, see small_int_to_float
+      const float drho = fmaf(__int_as_float(0x4B400000 + (int)w.rho[p]), cq, dq);
+      const float hp = __fsub_rn(t, h);
+      errmax = fmaxf(errmax, fabsf(fmaf(xp, hp, drho)));
+      const float y = __fmul_rn(xp, h), z = __fmul_rn(xp, hp);
+      z0 = __fadd_rn(z0, z);
       z1 = fmaf(z, j2f, z1);
-      z2 = fmaf(z, j2f * j2f, z2);
+      z2 = fmaf(z, __fmul_rn(j2f, j2f), z2);
       if (EXACT) {
         s0 = df_add_f(s0, y);
-        s3 = df_add_f(s3, y * j2f);
+        s3 = df_add_f(s3, __fmul_rn(y, j2f));
       } else {
-        s0.hi += y;
+        s0.hi = __fadd_rn(s0.hi, y);
         s3.hi = fmaf(y, j2f, s3.hi);
       }
       j2f = fmaf(2.f, jf, j2f + 1.f);  // (j + 1)^2
@@ -697,31 +751,48 @@ __device__ void pass_warp(const GridK& g, const FastGridK& fg, const FastWS& w,
       jz[8] += z2;
     }
   }
-  // warp totals of the J sums; lane k (mod 4) keeps row k of J:
-  // J[k][l] = vol d2^q m(p, q) for phi_k phi_l = v^p w^q
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) jz[i] += __shfl_xor_sync(FULL, jz[i], o);
-  }
+  // warp totals of the nine J sums and of ab1, scattered (recursive halving, the
+  // sums of a butterfly at half its instructions): lane bits 4..1 select one of
+  // sixteen slots, total i ends in lanes 2 rev(i) and 2 rev(i) + 1, rev the
+  // reversed four bits of i
+  float tot;
   {
-    const float vh = fg.vol_h, vd = vh * fg.d2q_h[1], vdd = vh * fg.d2q_h[2];
-    const float m00 = vh * jz[0], m10 = vh * jz[1], m20 = vh * jz[2], m30 = vh * jz[3],
-                m40 = vh * jz[4], m01 = vd * jz[5], m11 = vd * jz[6], m21 = vd * jz[7],
-                m02 = vdd * jz[8];
+    float v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = i < 9 ? jz[i] : (i == 9 ? ab1 : 0.f);
+#pragma unroll
+    for (int o = 16, n = 1; o >= 2; o >>= 1, n <<= 1) {
+      // slots of one parity of bit n stay here: pairs (i, i + n)
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int i = 0; i < 10; i += 2 * n) {
+        // (slots past the ninth are zeros; every lane takes part in every shuffle)
+        const float hi = i + n < 10 ? v[i + n] : 0.f;
+        const float send = up ? v[i] : hi, keep = up ? hi : v[i];
+        const float got = __shfl_xor_sync(FULL, send, o);
+        v[i] = keep + got;
+      }
+    }
+    tot = v[0] + __shfl_xor_sync(FULL, v[0], 1);
+  }
+  // lane k (mod 4) keeps row k of J: J[k][l] = vol d2^q m(p, q) for
+  // phi_k phi_l = v^p w^q, rows (1, v, w, v^2) times (1, v, w, v^2)
+  const float B1 = __shfl_sync(FULL, tot, 2 * 9);  // rev(9) = 9
+  {
+    // total i of this lane: i = rev(lane / 2); q = 1 for i = 5..7, 2 for i = 8
+    const int i = (int)(__brev((unsigned)lane >> 1) >> 28);
+    const float vh = fg.vol_h;
+    tot *= i < 5 ? vh : (i < 8 ? vh * fg.d2q_h[1] : vh * fg.d2q_h[2]);
+    // the lanes 2 rev(i) of the ten distinct entries of row k, by bytes:
+    // rows (m00 m10 m01 m20), (m10 m20 m11 m30), (m01 m11 m02 m21), (m20 m30 m21 m40)
     const int k = lane & 3;
-    // rows: (1, v, w, v^2) times (1, v, w, v^2)
-    o.J[0] = k == 0 ? m00 : (k == 1 ? m10 : (k == 2 ? m01 : m20));
-    o.J[1] = k == 0 ? m10 : (k == 1 ? m20 : (k == 2 ? m11 : m30));
-    o.J[2] = k == 0 ? m01 : (k == 1 ? m11 : (k == 2 ? m02 : m21));
-    o.J[3] = k == 0 ? m20 : (k == 1 ? m30 : (k == 2 ? m21 : m40));
+    const unsigned src = k == 0 ? 0x08141000u : (k == 1 ? 0x180C0810u : (k == 2 ? 0x1C020C14u : 0x041C1808u));
+#pragma unroll
+    for (int l = 0; l < 4; ++l) o.J[l] = __shfl_sync(FULL, tot, (src >> (8 * l)) & 31u);
   }
   // warp totals of the four sums, scattered (total k in lanes 8k..8k+7), in
   // double-float; then H_k in lane k and every total and H broadcast
   const df Ak = df_reduce_scatter4(a, lane);
-  float B1 = ab1;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) B1 += __shfl_xor_sync(FULL, B1, o);
   df A[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) A[k] = df{__shfl_sync(FULL, Ak.hi, 8 * k), __shfl_sync(FULL, Ak.lo, 8 * k)};
@@ -757,12 +828,9 @@ __device__ void pass_warp(const GridK& g, const FastGridK& fg, const FastWS& w,
   o.Habs[1] = vh * (fabsf(b.hi) * B1 + fabsf(c0.hi) * fabsf(A[0].hi));
   o.Habs[2] = vh * d2.hi * fabsf(A[3].hi);
   o.Habs[3] = vh * (bb.hi * fabsf(A[2].hi) + fabsf(c21.hi) * B1 + c00.hi * fabsf(A[0].hi));
-  float tm = tmax, em = errmax;
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    tm = fmaxf(tm, __shfl_xor_sync(FULL, tm, s));
-    em = fmaxf(em, __shfl_xor_sync(FULL, em, s));
-  }
+  // both >= 0: the order of the floats is that of their bits
+  const float tm = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(tmax)));
+  const float em = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(errmax)));
   o.tmax = tm * 1.000001f;  // the end points' FP32 rounding
   o.errmax = em;
   o.viol = em > e_hi;
@@ -1186,6 +1254,30 @@ __device__ __noinline__ void write_verbatim(const FusedArgs& a, long long b, dou
   __syncwarp();
 }
 
+// Largest finite value >= +0 of a row with negative, infinite or NaN values (or
+// -0, which counts as 0), and whether it holds any such value.
+struct RowMax {
+  unsigned long long umax;
+  int bad;
+};
+
+__device__ __noinline__ RowMax row_max_any(const double* xb, int P, int lane) {
+  unsigned long long umax = 0;
+  int bad = 0;
+#pragma unroll 1
+  for (int p = lane; p < P; p += 32) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(__ldg(xb + p));
+    if (u <= 0x7FEFFFFFFFFFFFFFull) umax = u > umax ? u : umax;
+    else bad |= u != 0x8000000000000000ull;
+  }
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const unsigned long long o = __shfl_xor_sync(FULL, umax, s);
+    umax = o > umax ? o : umax;
+  }
+  return {umax, __any_sync(FULL, bad)};
+}
+
 __device__ void fast_histogram(const FusedArgs& a, FastWS& w, long long b, int lane) {
   const GridK& g = a.grid;
   const ParamsK& pr = a.prm;
@@ -1198,30 +1290,38 @@ __device__ void fast_histogram(const FusedArgs& a, FastWS& w, long long b, int l
   // decoded row is fetched into L2 meanwhile, for the quantizer's loads
   for (int o = lane * 32; o < P; o += 32 * 32) asm volatile("prefetch.L2 [%0];" ::"l"(xhb + o));
   if (lane == 0) asm volatile("prefetch.L2 [%0];" ::"l"(xhb + P - 1));
-  unsigned long long umax = 0;
+  unsigned long long umax;
   int bad = 0;
-  // eight loads in flight per lane;
-  // a point past the end reads as +0
+  {
+    // the largest bit pattern as a signed word, and every sign bit: four
+    // instructions a value; a row with a sign bit, an infinity or a NaN takes
+    // the out-of-line scan.  Eight loads in flight per lane; a point past the
+    // end reads as +0.
+    long long m = 0;
+    unsigned sg = 0;
 #pragma unroll 1
-  for (int p0 = lane; p0 < P; p0 += 32 * 8) {
-    unsigned long long u[8];
+    for (int p0 = lane; p0 < P; p0 += 32 * 8) {
+      long long u[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int p = p0 + 32 * q;
-      u[q] = p < P ? (unsigned long long)__double_as_longlong(__ldg(xb + p)) : 0ull;
+      for (int q = 0; q < 8; ++q) {
+        const int p = p0 + 32 * q;
+        u[q] = p < P ? __double_as_longlong(__ldg(xb + p)) : 0ll;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        m = u[q] > m ? u[q] : m;
+        sg |= (unsigned)(u[q] >> 32);
+      }
     }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      if (u[q] <= 0x7FEFFFFFFFFFFFFFull) umax = u[q] > umax ? u[q] : umax;  // finite, >= +0
-      else bad |= u[q] != 0x8000000000000000ull;                            // -0 counts as 0
+    const unsigned mh = __reduce_max_sync(FULL, (unsigned)(m >> 32));
+    const unsigned ml = __reduce_max_sync(FULL, (unsigned)(m >> 32) == mh ? (unsigned)m : 0u);
+    umax = pack64(ml, mh);
+    if (__any_sync(FULL, (sg >> 31) != 0) || mh >= 0x7FF00000u) {
+      const RowMax r = row_max_any(xb, P, lane);
+      umax = r.umax;
+      bad = r.bad;
     }
   }
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    const unsigned long long o = __shfl_xor_sync(FULL, umax, s);
-    umax = o > umax ? o : umax;
-  }
-  bad = __any_sync(FULL, bad);
   const double s = __longlong_as_double((long long)umax);
   bool defer = bad || umax == 0;
   unsigned st = 0;
