@@ -45,7 +45,30 @@ using namespace dev;
 // Measured on the precision workload: sixteen warps in one CTA run 14 % faster
 // than the same sixteen warps as four CTAs of four (same registers, same
 // shared memory per warp, same histogram-to-SM mapping).
+//
+// What bounds the kernel is the supply of instructions: an SM partition issues
+// 64 % of its slots, and what costs time is code rather than warps.  Measured on
+// 262,144 histograms (39 x 39, tau = 1e-4), this form 3.91 ms:
+//  * 4.26 ms with 100 bytes of register spills in the 4 x 4 algebra; its
+//    constants now wait in shared memory (AlgWS) and the first column segment's
+//    sums in local memory, and nothing spills;
+//  * loops that outgrow the instruction buffers are slower: the quantizer's body
+//    is about 110 instructions (two rows a turn: 4.41 ms), the pass's about 30
+//    (two: 4.06, four: 4.10 ms);
+//  * more warps compete for the same buffers: twenty (96 registers, no spills)
+//    4.12 ms, twenty-four 4.08 ms;
+//  * two histograms a warp, their algebra side by side in half-warps and their
+//    points packed in FP32 pairs: 9.2 instead of 11.3 thousand instructions a
+//    histogram, but a body of 230, and 4.33 ms.
 constexpr int FW_MAX = 16;
+
+// The 4 x 4 algebra's constants of one histogram, in shared memory so that they
+// hold no registers during the passes.
+struct AlgWS {
+  float chol[16];  // L10 L20 L21 L30 L31 L32, 1 / L_kk, 1 / sqrt(M_kk)
+  float4 m[4][2];  // the rows of M: pairs (hi, lo)
+  float4 S, invS;
+};
 
 struct FastWS {
   float xp[AEQC_MAX_P];  // x' (float) for the Newton passes
@@ -55,6 +78,7 @@ struct FastWS {
       double ta[AEQC_MAX_NPAR], tb[AEQC_MAX_NPERP];  // exponential tables for f_out
     } t;
   };
+  AlgWS alg;
 };
 
 // float(v) for |v| < 2^22 without a conversion instruction (those issue to the
@@ -179,7 +203,6 @@ struct QConst {
   int k;
   int cx;    // floor(x 2^(QF-k)) = (mantissa << 10) >> (cx - E), E the exponent field
   int ch;    // trunc(xhat 2^(QF-k)) = (mantissa << 40) >> (ch - E)
-  int thr;   // exponent field of xhat at or above which |q| > 32766 for sure
 };
 
 // floor(log2(2 alpha fl(tau s))) for 2 alpha = 2^a2e and tau, s > 0 normal, on
@@ -217,8 +240,6 @@ __device__ __forceinline__ bool make_qconst(const ParamsK& pr, double s, int lev
   const int IBx = exponent_of(s) - c.k;  // s / Delta < 2^IBx
   c.cx = 1085 + c.k - QF;
   c.ch = 190 + c.k - QF;
-  // |xhat| >= 2^(61 - QF + k) = 2^23 Delta > s + 32766 Delta: certain escape
-  c.thr = 127 + 61 - QF + c.k;
   // x < 2^(IBx + QF) <= 2^60 units; Delta and the scale factors of the moment
   // sums (vol Delta 2^-30, vol Delta 2^-38) stay normal floats
   const bool ok = IBx >= 1 && IBx <= 22 && c.k - 64 >= -100 && c.k + 20 <= 100;
@@ -417,6 +438,18 @@ struct ColSums {
   float xs;
 };
 
+template <typename A, typename B>
+__device__ __forceinline__ void copy_sums(A& to, const B& from) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    to.b[q] = from.b[q];
+    to.a[q] = from.a[q];
+  }
+  to.u[0] = from.u[0];
+  to.u[1] = from.u[1];
+  to.xs = from.xs;
+}
+
 // a + b c for unsigned 32-bit b, c (one wide multiply-add)
 __device__ __forceinline__ unsigned long long mad_wide(unsigned long long a, unsigned b,
                                                        unsigned c) {
@@ -463,21 +496,17 @@ __device__ __forceinline__ void quant_segment(const Seg& sg, int n_par, const do
   int hard = 0;
   int nz = 0;
   int p = sg.j0 * n_par + sg.c;
-  // loads issued two points ahead of the work
+  // loads issued one row ahead of the work
   double xn = sg.j0 < sg.j1 ? __ldg(xb + p) : 0.0;
   float hn = sg.j0 < sg.j1 ? __ldg(xhb + p) : 0.f;
-  double xn2 = sg.j0 + 1 < sg.j1 ? __ldg(xb + p + n_par) : 0.0;
-  float hn2 = sg.j0 + 1 < sg.j1 ? __ldg(xhb + p + n_par) : 0.f;
   unsigned j2 = (unsigned)(sg.j0 * sg.j0);
 #pragma unroll 1
   for (int j = sg.j0; j < sg.j1; ++j, p += n_par) {
     const double x = xn;
     const float xh = hn;
-    xn = xn2;
-    hn = hn2;
-    if (j + 2 < sg.j1) {
-      xn2 = __ldg(xb + p + 2 * n_par);
-      hn2 = __ldg(xhb + p + 2 * n_par);
+    if (j + 1 < sg.j1) {
+      xn = __ldg(xb + p + n_par);
+      hn = __ldg(xhb + p + n_par);
     }
     const PointF o = quant_point_fast(x, xh, c);
     cb[p] = (int16_t)o.code;
@@ -516,6 +545,50 @@ __device__ __forceinline__ void quant_segment(const Seg& sg, int n_par, const do
   nonzero |= nz;
 }
 
+// v ic^r modulo 2^64: the even powers as unsigned words, the odd ones with a sign
+__device__ __forceinline__ unsigned long long times_ic(unsigned long long v, int i, int r) {
+  const unsigned e = (unsigned)(i * i);
+  if (r == 0) return v;
+  if (r == 2) return v * e;
+  if (r == 4) return v * (e * e);
+  return v * (unsigned long long)(long long)(r == 1 ? i : i * (int)e);
+}
+
+__device__ __forceinline__ float abs_v_sum(float xs1, float v1, float xs2, float v2) {
+  return fmaf(xs1, v1, __fmul_rn(xs2, v2));
+}
+
+// R, M and S from the polynomial moments mm (m00 m10 m20 m30 m40 m01 m11 m21
+// m02), the residual sums u over (1, ic, ic^2, j^2) in units of sr / vol and
+// S1 = sum |v| x'
+__device__ __forceinline__ void assemble_moments(const FastGridK& fg, df sr, const df (&mm)[9],
+                                                 const df (&u)[4], float S1, Moments& mo) {
+  const df b = {fg.coef_h[1][1], fg.coef_l[1][1]};   // C(1,1) b = b
+  const df c0 = {fg.coef_h[1][0], fg.coef_l[1][0]};  // C(1,0) c0 = c0
+  const df d2 = {fg.d2q_h[1], fg.d2q_l[1]};
+  // R_k = vol Delta 2^-38 sum phi_k rho, phi = (1, v, w, v^2), v = b ic + c0
+  mo.R[0] = df_mul(sr, u[0]);
+  mo.R[1] = df_mul(sr, df_add(df_mul(b, u[1]), df_mul(c0, u[0])));
+  mo.R[2] = df_mul(sr, df_mul(d2, u[3]));
+  {
+    const df cc[3] = {{fg.coef_h[2][0], fg.coef_l[2][0]},
+                      {fg.coef_h[2][1], fg.coef_l[2][1]},
+                      {fg.coef_h[2][2], fg.coef_l[2][2]}};
+    df acc = df_mul(cc[0], u[0]);
+    acc = df_add(acc, df_mul(cc[1], u[1]));
+    acc = df_add(acc, df_mul(cc[2], u[2]));
+    mo.R[3] = df_mul(sr, acc);
+  }
+  mo.M[0] = mm[0]; mo.M[1] = mm[1]; mo.M[2] = mm[5]; mo.M[3] = mm[2];
+  mo.M[4] = mm[2]; mo.M[5] = mm[6]; mo.M[6] = mm[3];
+  mo.M[7] = mm[8]; mo.M[8] = mm[7];
+  mo.M[9] = mm[4];
+  mo.S[0] = mm[0].hi;
+  mo.S[1] = fg.vol_h * S1;
+  mo.S[2] = mm[5].hi;
+  mo.S[3] = mm[2].hi;
+}
+
 // Quantize the histogram (row xb, decoded row xhb): codes to cb (global),
 // x' and the residual to shared memory, and the moments.
 __device__ void phase_a(const GridK& g, const FastGridK& fg, const double* xb,
@@ -525,38 +598,43 @@ __device__ void phase_a(const GridK& g, const FastGridK& fg, const double* xb,
   lane_segments(fg, g.n_par, g.n_perp, lane, sg1, sg2);
   int esc = 0, nonzero = 0;
   ColSums c1, c2;
-  quant_segment(sg1, g.n_par, xb, xhb, c, w, cb, c1, esc, nonzero);
-  quant_segment(sg2, g.n_par, xb, xhb, c, w, cb, c2, esc, nonzero);
+  {
+    // one copy of the walk for both segments; the first one's sums wait in local
+    // memory (volatile, or the compiler would keep 17 registers)
+    volatile ColSums keep;
+#pragma unroll 1
+    for (int part = 0; part < 2; ++part) {
+      Seg sg;
+      sg.c = part ? sg2.c : sg1.c;
+      sg.j0 = part ? sg2.j0 : sg1.j0;
+      sg.j1 = part ? sg2.j1 : sg1.j1;
+      quant_segment(sg, g.n_par, xb, xhb, c, w, cb, c2, esc, nonzero);
+      if (part == 0) copy_sums(keep, c2);
+    }
+    copy_sums(c1, keep);
+  }
   // fold with the powers of i - i_c: U_q over weights 1, ic, ic^2, j^2 and T
   // over (ic^r j^(2q)) in the order T00 T10 T20 T30 T40 T01 T11 T21 T02, the
   // latter as Tb + 2^32 Ta (totals below 2^63)
   long long U[4], Tb[9], Ta[9];
   {
-    // v ic^r: the even powers as unsigned words, the odd ones with a sign
     const int i1 = sg1.c - fg.i_c, i2 = sg2.c - fg.i_c;
-    auto times = [](unsigned long long v, int i, int r) -> unsigned long long {
-      const unsigned e = (unsigned)(i * i);
-      if (r == 0) return v;
-      if (r == 2) return v * e;
-      if (r == 4) return v * (e * e);
-      return v * (unsigned long long)(long long)(r == 1 ? i : i * (int)e);
-    };
     const int rq[9][2] = {{0, 0}, {1, 0}, {2, 0}, {3, 0}, {4, 0}, {0, 1}, {1, 1}, {2, 1}, {0, 2}};
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
       const int r = rq[k][0], q = rq[k][1];
-      Tb[k] = (long long)(times(c1.b[q], i1, r) + times(c2.b[q], i2, r));
-      Ta[k] = (long long)(times(c1.a[q], i1, r) + times(c2.a[q], i2, r));
+      Tb[k] = (long long)(times_ic(c1.b[q], i1, r) + times_ic(c2.b[q], i2, r));
+      Ta[k] = (long long)(times_ic(c1.a[q], i1, r) + times_ic(c2.a[q], i2, r));
     }
     const unsigned long long u1 = (unsigned long long)rho_sum(c1, 0),
                              u2 = (unsigned long long)rho_sum(c2, 0);
 #pragma unroll
-    for (int r = 0; r < 3; ++r) U[r] = (long long)(times(u1, i1, r) + times(u2, i2, r));
+    for (int r = 0; r < 3; ++r) U[r] = (long long)(times_ic(u1, i1, r) + times_ic(u2, i2, r));
     U[3] = rho_sum(c1, 1) + rho_sum(c2, 1);
   }
-  const float b_f = fg.b_f, c0_f = fg.c0_f;
-  float s1 = c1.xs * fabsf(fmaf(b_f, small_int_to_float(sg1.c - fg.i_c), c0_f)) +
-             c2.xs * fabsf(fmaf(b_f, small_int_to_float(sg2.c - fg.i_c), c0_f));
+  const float s1 = abs_v_sum(
+      c1.xs, fabsf(fmaf(fg.b_f, small_int_to_float(sg1.c - fg.i_c), fg.c0_f)), c2.xs,
+      fabsf(fmaf(fg.b_f, small_int_to_float(sg2.c - fg.i_c), fg.c0_f)));
   __syncwarp();
   // exact warp totals (the host bounds them below 2^63), scattered over the
   // lanes: lane k holds total k of (U0..U3, Tb0..Tb8, Ta0..Ta8); each lane
@@ -595,31 +673,7 @@ __device__ void phase_a(const GridK& g, const FastGridK& fg, const double* xb,
   for (int j = 0; j < 9; ++j) mm[j] = df{__shfl_sync(FULL, mj.hi, j), __shfl_sync(FULL, mj.lo, j)};
 #pragma unroll
   for (int q = 0; q < 4; ++q) u[q] = df{__shfl_sync(FULL, mine.hi, q), __shfl_sync(FULL, mine.lo, q)};
-  const df b = {fg.coef_h[1][1], fg.coef_l[1][1]};   // C(1,1) b = b
-  const df c0 = {fg.coef_h[1][0], fg.coef_l[1][0]};  // C(1,0) c0 = c0
-  const df d2 = {fg.d2q_h[1], fg.d2q_l[1]};
-  // R_k = vol Delta 2^-38 sum phi_k rho, phi = (1, v, w, v^2), v = b ic + c0
-  mo.R[0] = df_mul(sr, u[0]);
-  mo.R[1] = df_mul(sr, df_add(df_mul(b, u[1]), df_mul(c0, u[0])));
-  mo.R[2] = df_mul(sr, df_mul(d2, u[3]));
-  {
-    const df cc[3] = {{fg.coef_h[2][0], fg.coef_l[2][0]},
-                      {fg.coef_h[2][1], fg.coef_l[2][1]},
-                      {fg.coef_h[2][2], fg.coef_l[2][2]}};
-    df acc = df_mul(cc[0], u[0]);
-    acc = df_add(acc, df_mul(cc[1], u[1]));
-    acc = df_add(acc, df_mul(cc[2], u[2]));
-    mo.R[3] = df_mul(sr, acc);
-  }
-  // mm: m00 m10 m20 m30 m40 m01 m11 m21 m02
-  mo.M[0] = mm[0]; mo.M[1] = mm[1]; mo.M[2] = mm[5]; mo.M[3] = mm[2];
-  mo.M[4] = mm[2]; mo.M[5] = mm[6]; mo.M[6] = mm[3];
-  mo.M[7] = mm[8]; mo.M[8] = mm[7];
-  mo.M[9] = mm[4];
-  mo.S[0] = mm[0].hi;
-  mo.S[1] = fg.vol_h * S1;
-  mo.S[2] = mm[5].hi;
-  mo.S[3] = mm[2].hi;
+  assemble_moments(fg, sr, mm, u, S1, mo);
   mo.flags = 0;
   if (__any_sync(FULL, esc)) mo.flags |= AEQC_ST_CODE_ESCAPE;
   if (!__any_sync(FULL, nonzero)) mo.flags |= AEQC_ST_AE_EXACT;
@@ -657,6 +711,40 @@ __device__ __forceinline__ TCoef make_tcoef(const FastGridK& fg, const df lam[4]
   t.h[2] = a2.hi; t.l[2] = a2.lo;
   t.h[3] = a3.hi; t.l[3] = a3.lo;
   return t;
+}
+
+// H_k = vol sum phi_k y from the sums A of y, y ic, y ic^2, y j^2, with
+// phi = (1, v, w, v^2), v = b ic + c0, w = d2 j^2:
+// H0 = vol A0, H1 = vol (b A1 + c0 A0), H2 = vol d2 A3,
+// H3 = vol (b^2 A2 + 2 b c0 A1 + c0^2 A0); the lane's own k: as
+// vol (a0 A0 + a1 A1 + a2 A2 + a3 A3) with per-lane coefficients (1,0,0,0),
+// (c0,b,0,0), (0,0,0,d2), (c0^2,2bc0,b^2,0), without divergence
+__device__ __forceinline__ df h_row(const FastGridK& fg, const df (&A)[4], int k) {
+  const df vol = {fg.vol_h, fg.vol_l};
+  const df zero = {0.f, 0.f};
+  const df a0 = k == 0 ? df{1.f, 0.f}
+                       : (k == 1 ? df{fg.coef_h[1][0], fg.coef_l[1][0]}
+                                 : (k == 3 ? df{fg.coef_h[2][0], fg.coef_l[2][0]} : zero));
+  const df a1 = k == 1 ? df{fg.coef_h[1][1], fg.coef_l[1][1]}
+                       : (k == 3 ? df{fg.coef_h[2][1], fg.coef_l[2][1]} : zero);
+  const df a2 = k == 3 ? df{fg.coef_h[2][2], fg.coef_l[2][2]} : zero;
+  const df a3 = k == 2 ? df{fg.d2q_h[1], fg.d2q_l[1]} : zero;
+  df acc = df_add(df_mul(a0, A[0]), df_mul(a1, A[1]));
+  acc = df_add(acc, df_add(df_mul(a2, A[2]), df_mul(a3, A[3])));
+  return df_mul(vol, acc);
+}
+
+// Bounds of the sums of |terms| of H (B1 = sum |ic| y)
+__device__ __forceinline__ void h_abs(const FastGridK& fg, const df (&A)[4], float B1, PassOut& o) {
+  const df c0 = {fg.coef_h[1][0], fg.coef_l[1][0]}, b = {fg.coef_h[1][1], fg.coef_l[1][1]};
+  const df c00 = {fg.coef_h[2][0], fg.coef_l[2][0]}, c21 = {fg.coef_h[2][1], fg.coef_l[2][1]};
+  const df bb = {fg.coef_h[2][2], fg.coef_l[2][2]}, d2 = {fg.d2q_h[1], fg.d2q_l[1]};
+  // y >= 0 (h >= 0, x' >= 0), so A0, A2, A3 are sums of non-negative terms
+  const float vh = fg.vol_h;
+  o.Habs[0] = vh * fabsf(A[0].hi);
+  o.Habs[1] = vh * (fabsf(b.hi) * B1 + fabsf(c0.hi) * fabsf(A[0].hi));
+  o.Habs[2] = vh * d2.hi * fabsf(A[3].hi);
+  o.Habs[3] = vh * (bb.hi * fabsf(A[2].hi) + fabsf(c21.hi) * B1 + c00.hi * fabsf(A[0].hi));
 }
 
 // One pass at lambda: H(lambda) and the end-to-end check.  EXACT selects
@@ -700,6 +788,7 @@ __device__ void pass_warp(const GridK& g, const FastGridK& fg, const FastWS& w,
     // rounding is written out: the step counts must not depend on contraction.
     float jf = j0f, j2f = j0f * j0f;
     int p = sgm.j0 * g.n_par + sgm.c;
+#pragma unroll 1
     for (int j = sgm.j0; j < sgm.j1; ++j, p += g.n_par) {
       const float t = __fadd_rn(fmaf(tc.h[2], j2f, ah), fmaf(tc.l[2], j2f, al));
       const float xp = w.xp[p];
@@ -796,38 +885,10 @@ __device__ void pass_warp(const GridK& g, const FastGridK& fg, const FastWS& w,
   df A[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) A[k] = df{__shfl_sync(FULL, Ak.hi, 8 * k), __shfl_sync(FULL, Ak.lo, 8 * k)};
-  const df vol = {fg.vol_h, fg.vol_l};
-  // H_k = vol sum phi_k y with phi = (1, v, w, v^2), v = b ic + c0, w = d2 j^2:
-  // H0 = vol A0, H1 = vol (b A1 + c0 A0), H2 = vol d2 A3,
-  // H3 = vol (b^2 A2 + 2 b c0 A1 + c0^2 A0); lane k forms H_k
-  df hk;
-  {
-    // H_k = vol (a0 A0 + a1 A1 + a2 A2 + a3 A3) with per-lane coefficients
-    // (1,0,0,0), (c0,b,0,0), (0,0,0,d2), (c0^2,2bc0,b^2,0): no divergence
-    const int k = lane & 3;
-    const df zero = {0.f, 0.f};
-    const df a0 = k == 0 ? df{1.f, 0.f}
-                         : (k == 1 ? df{fg.coef_h[1][0], fg.coef_l[1][0]}
-                                   : (k == 3 ? df{fg.coef_h[2][0], fg.coef_l[2][0]} : zero));
-    const df a1 = k == 1 ? df{fg.coef_h[1][1], fg.coef_l[1][1]}
-                         : (k == 3 ? df{fg.coef_h[2][1], fg.coef_l[2][1]} : zero);
-    const df a2 = k == 3 ? df{fg.coef_h[2][2], fg.coef_l[2][2]} : zero;
-    const df a3 = k == 2 ? df{fg.d2q_h[1], fg.d2q_l[1]} : zero;
-    df acc = df_add(df_mul(a0, A[0]), df_mul(a1, A[1]));
-    acc = df_add(acc, df_add(df_mul(a2, A[2]), df_mul(a3, A[3])));
-    hk = df_mul(vol, acc);
-  }
+  const df hk = h_row(fg, A, lane & 3);
 #pragma unroll
   for (int k = 0; k < 4; ++k) o.H[k] = df{__shfl_sync(FULL, hk.hi, k), __shfl_sync(FULL, hk.lo, k)};
-  const df c0 = {fg.coef_h[1][0], fg.coef_l[1][0]}, b = {fg.coef_h[1][1], fg.coef_l[1][1]};
-  const df c00 = {fg.coef_h[2][0], fg.coef_l[2][0]}, c21 = {fg.coef_h[2][1], fg.coef_l[2][1]};
-  const df bb = {fg.coef_h[2][2], fg.coef_l[2][2]}, d2 = {fg.d2q_h[1], fg.d2q_l[1]};
-  // y >= 0 (h >= 0, x' >= 0), so A0, A2, A3 are sums of non-negative terms
-  const float vh = fg.vol_h;
-  o.Habs[0] = vh * fabsf(A[0].hi);
-  o.Habs[1] = vh * (fabsf(b.hi) * B1 + fabsf(c0.hi) * fabsf(A[0].hi));
-  o.Habs[2] = vh * d2.hi * fabsf(A[3].hi);
-  o.Habs[3] = vh * (bb.hi * fabsf(A[2].hi) + fabsf(c21.hi) * B1 + c00.hi * fabsf(A[0].hi));
+  h_abs(fg, A, B1, o);
   // both >= 0: the order of the floats is that of their bits
   const float tm = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(tmax)));
   const float em = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(errmax)));
@@ -906,47 +967,216 @@ __device__ __forceinline__ void chol_solve(const Chol& ch, const float r[4], flo
   for (int k = 0; k < 4; ++k) dlt[k] = z[k] * ch.d[k];
 }
 
+__device__ __forceinline__ float inv_s(float S) { return S > 1e-30f ? 1.f / S : 1e30f; }
+
+// The factor, the rows of M, S and 1 / S to shared memory (every lane holds them
+// all and writes the same values)
+__device__ __forceinline__ void store_algebra(const Moments& mo, const Chol& ch, AlgWS& w) {
+  float4* c = reinterpret_cast<float4*>(w.chol);
+  __syncwarp();
+  c[0] = make_float4(ch.L[1][0], ch.L[2][0], ch.L[2][1], ch.L[3][0]);
+  c[1] = make_float4(ch.L[3][1], ch.L[3][2], ch.inv[0], ch.inv[1]);
+  c[2] = make_float4(ch.inv[2], ch.inv[3], ch.d[0], ch.d[1]);
+  c[3] = make_float4(ch.d[2], ch.d[3], 0.f, 0.f);
+  const int idx[4][4] = {{0, 1, 2, 3}, {1, 4, 5, 6}, {2, 5, 7, 8}, {3, 6, 8, 9}};
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const df p = mo.M[idx[k][2 * h]], q = mo.M[idx[k][2 * h + 1]];
+      w.m[k][h] = make_float4(p.hi, p.lo, q.hi, q.lo);
+    }
+  w.S = make_float4(mo.S[0], mo.S[1], mo.S[2], mo.S[3]);
+  w.invS = make_float4(inv_s(mo.S[0]), inv_s(mo.S[1]), inv_s(mo.S[2]), inv_s(mo.S[3]));
+  __syncwarp();
+}
+
+// a volatile 16-byte read: stays where it is written, so that no register holds
+// the value across a pass
+__device__ __forceinline__ float4 lds4(const void* p) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"((unsigned)__cvta_generic_to_shared(p)));
+  return v;
+}
+__device__ __forceinline__ void load4(const float4& p, float (&o)[4]) {
+  const float4 v = lds4(&p);
+  o[0] = v.x;
+  o[1] = v.y;
+  o[2] = v.z;
+  o[3] = v.w;
+}
+__device__ __forceinline__ void load_row(const AlgWS& w, int kr, df (&row)[4]) {
+  const float4 a = lds4(&w.m[kr][0]), b = lds4(&w.m[kr][1]);
+  row[0] = df{a.x, a.y};
+  row[1] = df{a.z, a.w};
+  row[2] = df{b.x, b.y};
+  row[3] = df{b.z, b.w};
+}
+__device__ __forceinline__ void load_chol(const AlgWS& w, Chol& ch) {
+  const float4* c = reinterpret_cast<const float4*>(w.chol);
+  const float4 a = lds4(c), b = lds4(c + 1), d = lds4(c + 2), e = lds4(c + 3);
+  ch.L[1][0] = a.x;
+  ch.L[2][0] = a.y;
+  ch.L[2][1] = a.z;
+  ch.L[3][0] = a.w;
+  ch.L[3][1] = b.x;
+  ch.L[3][2] = b.y;
+  ch.inv[0] = b.z;
+  ch.inv[1] = b.w;
+  ch.inv[2] = d.x;
+  ch.inv[3] = d.y;
+  ch.d[0] = d.z;
+  ch.d[1] = d.w;
+  ch.d[2] = e.x;
+  ch.d[3] = e.y;
+}
+__device__ __forceinline__ float lds1(const float* p) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"((unsigned)__cvta_generic_to_shared(p)));
+  return v;
+}
+__device__ __forceinline__ void chol_solve(const AlgWS& w, const float r[4], float dlt[4]) {
+  Chol ch;
+  load_chol(w, ch);
+  chol_solve(ch, r, dlt);
+}
+
 struct NewtonState {
   int check_viol;  // end-to-end violation at the final lambda (valid when converged)
   float gres[4];   // |g_k| / S_k at the final lambda
 };
 
+// Error budget of g (absolute, per moment k), so that "converged" proves
+// |g_k| <= tol S_k with S_k = sum vol |phi_k| f at the final lambda:
+//  * moments: the residual is summed in units of Delta 2^-38 within two
+//    units per point, x' within one unit (its error enters as M lambda):
+//    Delta wk (2^-37 + 2^-38 tb), wk = vol sum |phi_k| over the grid;
+//  * the double-float assembly of g: below 2e-15 S_k;
+//  * H (after a pass, a bound on sum vol |phi_k| |x' h| in Habs):
+//    summation <= 3.5e-6 Habs in FP32 (none with TwoSum accumulation);
+//    terms: x' to float (2^-23), t to float (|dt| <= 2.1 u |t| + 2^-43 tb,
+//    |h'(t)| <= 1.06 |t|: 4.7 u relative to h), h's polynomial in FP32:
+//    <= 8e-7 Habs + 1.2e-13 tb tmax S_k; the series for h cut after t^5:
+//    |t|^6 e^|t| / 720 <= 0.003 t^4 h(t) for |t| <= 0.05;
+//  * S_k at f is at least S_k(x') (1 - tmax).
+// The budget is kept as one number, max_k err_k / S_k.
+
+// tb: a bound of |lambda.phi| on the grid
+__device__ __forceinline__ float t_bound(const FastGridK& fg, const df* lam) {
+  return fabsf(lam[0].hi) + fabsf(lam[1].hi) * fg.vmax + fabsf(lam[2].hi) * fg.wmax +
+         fabsf(lam[3].hi) * fg.vmax * fg.vmax;
+}
+
+__device__ __forceinline__ float moment_error(const FastGridK& fg, float dl_f, float tb,
+                                              const float (&invS)[4]) {
+  float erel = 2e-15f;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    erel = fmaxf(erel, fg.wk[k] * dl_f * fmaf(3.7e-12f, tb, 7.3e-12f) * invS[k] + 2e-15f);
+  return erel;
+}
+
+// FP32 rounding of the check (x' e^{-t} - x evaluated as x'(h - t) - Delta rho)
+// plus the 2^-15 Delta fixed point of rho
+__device__ __forceinline__ float check_margin(float s, float tb, float dl_f) {
+  return 4e-7f * (s * tb + dl_f) + 3.0517578125e-05f * dl_f + 1e-30f;
+}
+
+// The FP32 sums of H need TwoSum accumulation: their error bound (<= 50 FP32
+// roundings per lane: 50 u sum|terms|) is too wide
+__device__ __forceinline__ bool pass_imprecise(const PassOut& po, const float (&S)[4]) {
+  bool redo = false;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) redo = redo || 3.5e-6f * po.Habs[k] > 1e-13f * S[k];
+  return redo;
+}
+
+__device__ __forceinline__ float pass_error(const PassOut& po, bool redo, float tb,
+                                            const float (&invS)[4]) {
+  const float t2 = po.tmax * po.tmax;
+  const float hrel = (redo ? 8e-7f : 4.3e-6f) + 0.003f * t2 * t2;
+  float eh = 0.f;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) eh = fmaxf(eh, hrel * po.Habs[k] * invS[k]);
+  return eh + 1.2e-13f * tb * po.tmax;
+}
+
+__device__ __forceinline__ float residual_k(float g, float invS, float sf, float floor_r) {
+  return fabsf(g) * invS * sf + floor_r;
+}
+
+// Certificate after a pass (unit step d = d1 + d2 + d3): in row k,
+//   g_k(l + d) = (g - M dd)_k + (J dd - M d3 + J d3)_k + e_J + R2_k,
+// the first term in double-float, the second in FP32 (roundings within
+// 1e-6 of the sum of the magnitudes of its products, which also covers
+// dd's rounding of d1 + d2); e_J, the FP32 error of J, is below
+// 1e-5 tmax e^tmax tb_d S_k (|h'(t)| <= |t| e^|t|, about 70 roundings
+// per sum; tb_d bounds |d.phi| on the grid); the remainder of the
+// expansion is |R2_k| <= e^tt tb_d^2 S_k / 2 (h'' = e^-t, tt = tmax + tb_d).
+// g itself carries at most err_k (the budget above, its x' term widened
+// to the new lambda), and S_k at the new f is at least S_k (1 - tt).  The
+// pointwise check moves by at most x'max e^tmax (e^tb_d - 1).  When both
+// bounds hold, the step is taken and the histogram converged without the
+// pass at the new lambda.
+struct Certificate {
+  float rel;          // bound of |g_k| / S_k at the new lambda, k the lane's row
+  bool small, check;  // tt in range; the pointwise check holds
+};
+
+__device__ __forceinline__ Certificate certify(const FastGridK& fg, const AlgWS& alg,
+                                               const float (&Jr)[4], int kr, df rd1,
+                                               const float (&d1)[4], const float (&d2)[4],
+                                               const float (&d3)[4], const float (&dd)[4],
+                                               float vk, float tmax, float errmax, float pmargin,
+                                               float erel, float dl_f, float s, float e) {
+  float dn[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) dn[k] = dd[k] + d3[k];
+  const float tbd = (fabsf(dn[0]) + fabsf(dn[1]) * fg.vmax + fabsf(dn[2]) * fg.wmax +
+                     fabsf(dn[3]) * fg.vmax * fg.vmax) *
+                    1.000001f;
+  const float tt = tmax + tbd;
+  const float grow = (1.f + 1.1f * tt) * 1.01f;  // e^tt for tt < 0.05, padded
+  // residual of the solve, row k in lane k: g - M dd = (g - M d1) - M d2,
+  // the second product in FP32 (|d2| ~ 1e-6 |d1|; its rounding in cabs)
+  df rowM[4];
+  load_row(alg, kr, rowM);
+  const float Sk = lds1(reinterpret_cast<const float*>(&alg.S) + kr),
+              iSk = lds1(reinterpret_cast<const float*>(&alg.invS) + kr);
+  float rs = rd1.hi, corr = vk + rd1.lo, cabs = 0.f;
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    rs = fmaf(-rowM[l].hi, d2[l], rs);
+    corr = fmaf(Jr[l] - rowM[l].hi, d3[l], corr);
+    cabs = fmaf(fabsf(Jr[l]) + fabsf(rowM[l].hi), fabsf(dd[l]) + fabsf(d2[l]) + fabsf(d3[l]),
+                cabs);
+  }
+  cabs += fabsf(rs);
+  const float ek = erel * Sk +
+                   3.7e-12f * dl_f * tbd *
+                       (kr == 0 ? fg.wk[0] : (kr == 1 ? fg.wk[1] : (kr == 2 ? fg.wk[2] : fg.wk[3]))) +
+                   1e-6f * cabs + Sk * grow * tbd * fmaf(1e-5f, tmax, 0.5f * tbd);
+  const float bk = fabsf(rs + corr) + ek;
+  Certificate c;
+  c.rel = bk * iSk * fmaf(1.06f, tt, 1.f);
+  c.small = tt < 0.05f;
+  const float xpmax = s + 2.f * dl_f;
+  c.check = errmax + pmargin + xpmax * grow * tbd * 1.01f <= e;
+  return c;
+}
+
 // Round 1 of Eq. (6) with the chord Jacobian M from lam (in/out).
 // Returns 1 converged, 0 not converged, -1 defer (precision guards).
 __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
-                           const QConst& c, const Moments& mo, const Chol& ch, df lam[4],
+                           const QConst& c, df Rk, df lam[4],
                            int max_iter, float step, float tol, float e, float s, int* iters,
                            float* r0, float* rlast, NewtonState& ns, int lane) {
   // lane k (mod 4) owns row k of M and component k of R: the matrix-vector
   // products run one row per lane and are gathered by shuffles
   const int kr = lane & 3;
-  df rowM[4];
-  {
-    const int idx[4][4] = {{0, 1, 2, 3}, {1, 4, 5, 6}, {2, 5, 7, 8}, {3, 6, 8, 9}};
-#pragma unroll
-    for (int l = 0; l < 4; ++l)
-      rowM[l] = kr == 0 ? mo.M[idx[0][l]]
-                        : (kr == 1 ? mo.M[idx[1][l]] : (kr == 2 ? mo.M[idx[2][l]] : mo.M[idx[3][l]]));
-  }
-  const df Rk = kr == 0 ? mo.R[0] : (kr == 1 ? mo.R[1] : (kr == 2 ? mo.R[2] : mo.R[3]));
-  // 1 / S_k once per histogram: the residual tests multiply
-  float invS[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) invS[k] = mo.S[k] > 1e-30f ? 1.f / mo.S[k] : 1e30f;
-  // Error budget of g (absolute, per moment k), so that "converged" proves
-  // |g_k| <= tol S_k with S_k = sum vol |phi_k| f at the final lambda:
-  //  * moments: the residual is summed in units of Delta 2^-38 within two
-  //    units per point, x' within one unit (its error enters as M lambda):
-  //    Delta wk (2^-37 + 2^-38 tb), wk = vol sum |phi_k| over the grid;
-  //  * the double-float assembly of g: below 2e-15 S_k;
-  //  * H (after a pass, a bound on sum vol |phi_k| |x' h| in Habs):
-  //    summation <= 3.5e-6 Habs in FP32 (none with TwoSum accumulation);
-  //    terms: x' to float (2^-23), t to float (|dt| <= 2.1 u |t| + 2^-43 tb,
-  //    |h'(t)| <= 1.06 |t|: 4.7 u relative to h), h's polynomial in FP32:
-  //    <= 8e-7 Habs + 1.2e-13 tb tmax S_k; the series for h cut after t^5:
-  //    |t|^6 e^|t| / 720 <= 0.003 t^4 h(t) for |t| <= 0.05;
-  //  * S_k at f is at least S_k(x') (1 - tmax).
-  // The budget is kept as one number, max_k err_k / S_k.
+  const AlgWS& alg = w.alg;
   bool force_pass = false;  // converged at lambda = 0: repeat the iteration with the check
   float erel = 0.f;
   for (int it = 0;; ++it) {
@@ -957,40 +1187,37 @@ __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
     int viol = 0, unc = 0;
     bool did_pass = false;
     float tmax = 0.f, errmax = 0.f, pmargin = 0.f;
-    const float tb = fabsf(lam[0].hi) + fabsf(lam[1].hi) * fg.vmax + fabsf(lam[2].hi) * fg.wmax +
-                     fabsf(lam[3].hi) * fg.vmax * fg.vmax;
-    erel = 2e-15f;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      erel = fmaxf(erel, fg.wk[k] * c.dl_f * fmaf(3.7e-12f, tb, 7.3e-12f) * invS[k] + 2e-15f);
+    const float tb = t_bound(fg, lam);
+    {
+      float invS[4];
+      load4(alg.invS, invS);
+      erel = moment_error(fg, c.dl_f, tb, invS);
+    }
     auto do_pass = [&]() {
-      // FP32 rounding of the check (x' e^{-t} - x evaluated as x'(h - t) - Delta rho)
-      // plus the 2^-15 Delta fixed point of rho
-      const float margin = 4e-7f * (s * tb + c.dl_f) + 3.0517578125e-05f * c.dl_f + 1e-30f;
+      const float margin = check_margin(s, tb, c.dl_f);
       PassOut po;
       const TCoef tc = make_tcoef(fg, lam);
       // FP32 sums first; again with TwoSum accumulation when their error bound
-      // (<= 50 FP32 roundings per lane: 50 u sum|terms|) is too wide.  One
-      // call site for both (the kernel is bound by instruction fetch).
+      // is too wide.  One call site for both (the kernel is bound by instruction
+      // fetch).
       bool redo = false;
 #pragma unroll 1
       for (int rep = 0; rep < 2; ++rep) {
         pass_warp(g, fg, w, c, tc, e - margin, e + margin, po, lane, rep != 0);
         if (rep) break;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) redo = redo || 3.5e-6f * po.Habs[k] > 1e-13f * mo.S[k];
+        float S[4];
+        load4(alg.S, S);
+        redo = pass_imprecise(po, S);
         if (!redo) break;
       }
-      const float t2 = po.tmax * po.tmax;
-      const float hrel = (redo ? 8e-7f : 4.3e-6f) + 0.003f * t2 * t2;
-      float eh = 0.f;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         H[k] = po.H[k];
         Jr[k] = po.J[k];
-        eh = fmaxf(eh, hrel * po.Habs[k] * invS[k]);
       }
-      erel += eh + 1.2e-13f * tb * po.tmax;
+      float invS[4];
+      load4(alg.invS, invS);
+      erel += pass_error(po, redo, tb, invS);
       viol = po.viol;
       unc = po.uncertain;
       did_pass = true;
@@ -1005,6 +1232,8 @@ __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
     {
       df gl = df_neg(Rk);
       if (!zero_lam) {
+        df rowM[4];
+        load_row(alg, kr, rowM);
         df ml = df_mul(rowM[0], lam[0]);
 #pragma unroll
         for (int l = 1; l < 4; ++l) ml = df_add(ml, df_mul(rowM[l], lam[l]));
@@ -1022,9 +1251,12 @@ __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
     const float floor_r = erel * sf;
     float res = 0.f;
     bool finite_ok = true;
+    float invS[4], S[4];
+    load4(alg.invS, invS);
+    load4(alg.S, S);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const float rk = fabsf(gk[k].hi) * invS[k] * sf + floor_r;
+      const float rk = residual_k(gk[k].hi, invS[k], sf, floor_r);
       finite_ok = finite_ok && isfinite(rk);
       ns.gres[k] = rk;
       res = fmaxf(res, rk);
@@ -1036,7 +1268,7 @@ __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
     if (tmax > 0.05f || floor_r > 0.5f * tol) return -1;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if (fabsf(H[k].hi) > 1e-5f * mo.S[k]) return -1;
+      if (fabsf(H[k].hi) > 1e-5f * S[k]) return -1;
     if (res <= tol) {
       if (!did_pass) {  // lambda = 0 converged: still check every point
         force_pass = true;
@@ -1055,7 +1287,7 @@ __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
     float r[4], d1[4], d2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int k = 0; k < 4; ++k) r[k] = gk[k].hi;
-    chol_solve(ch, r, d1);
+    chol_solve(alg, r, d1);
     if (zero_lam) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) lam[k] = df{step * d1[k], 0.f};
@@ -1063,6 +1295,8 @@ __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
     }
     df rd1;  // g - M d1 in row kr (double-float), reused by the certificate
     {
+      df rowM[4];
+      load_row(alg, kr, rowM);
       df md = df_mul_f(rowM[0], d1[0]);
 #pragma unroll
       for (int l = 1; l < 4; ++l) md = df_add(md, df_mul_f(rowM[l], d1[l]));
@@ -1072,7 +1306,7 @@ __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
 #pragma unroll
       for (int k = 0; k < 4; ++k) r[k] = __shfl_sync(FULL, rl, k);
     }
-    chol_solve(ch, r, d2);
+    chol_solve(alg, r, d2);
     // Newton correction from the Jacobian of H that the pass measured:
     // g(l + d) = g(l) - M d + J d + R2 with J = sum vol phi phi^T x' h'(t), so
     // d3 = M^-1 (J (d1 + d2)) makes d1 + d2 + d3 solve (M - J) d = g up to
@@ -1086,68 +1320,26 @@ __device__ int round1_fast(const GridK& g, const FastGridK& fg, const FastWS& w,
       vk = fmaf(Jr[3], dd[3], fmaf(Jr[2], dd[2], fmaf(Jr[1], dd[1], Jr[0] * dd[0])));
 #pragma unroll
       for (int k = 0; k < 4; ++k) r[k] = __shfl_sync(FULL, vk, k);
-      chol_solve(ch, r, d3);
+      chol_solve(alg, r, d3);
     }
-    // Certificate after a pass (unit step d = d1 + d2 + d3): in row k,
-    //   g_k(l + d) = (g - M dd)_k + (J dd - M d3 + J d3)_k + e_J + R2_k,
-    // the first term in double-float, the second in FP32 (roundings within
-    // 1e-6 of the sum of the magnitudes of its products, which also covers
-    // dd's rounding of d1 + d2); e_J, the FP32 error of J, is below
-    // 1e-5 tmax e^tmax tb_d S_k (|h'(t)| <= |t| e^|t|, about 70 roundings
-    // per sum; tb_d bounds |d.phi| on the grid); the remainder of the
-    // expansion is |R2_k| <= e^tt tb_d^2 S_k / 2 (h'' = e^-t, tt = tmax + tb_d).
-    // g itself carries at most err_k (the budget above, its x' term widened
-    // to the new lambda), and S_k at the new f is at least S_k (1 - tt).  The
-    // pointwise check moves by at most x'max e^tmax (e^tb_d - 1).  When both
-    // bounds hold, the step is taken and the histogram converged without the
-    // pass at the new lambda.
     if (did_pass && step == 1.f && !viol && !unc) {
-      float dn[4];
+      const Certificate cf = certify(fg, alg, Jr, kr, rd1, d1, d2, d3, dd, vk, tmax,
+                                     errmax, pmargin, erel, c.dl_f, s, e);
+      float worst = cf.rel;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) dn[k] = dd[k] + d3[k];
-      const float tbd = (fabsf(dn[0]) + fabsf(dn[1]) * fg.vmax + fabsf(dn[2]) * fg.wmax +
-                         fabsf(dn[3]) * fg.vmax * fg.vmax) *
-                        1.000001f;
-      const float tt = tmax + tbd;
-      if (tt < 0.05f) {
-        const float grow = (1.f + 1.1f * tt) * 1.01f;  // e^tt for tt < 0.05, padded
-        // residual of the solve, row k in lane k: g - M dd = (g - M d1) - M d2,
-        // the second product in FP32 (|d2| ~ 1e-6 |d1|; its rounding in cabs)
-        const float Sk = kr == 0 ? mo.S[0] : (kr == 1 ? mo.S[1] : (kr == 2 ? mo.S[2] : mo.S[3]));
-        float rs = rd1.hi, corr = vk + rd1.lo, cabs = 0.f;
+      for (int o = 1; o < 4; o <<= 1) worst = fmaxf(worst, __shfl_xor_sync(FULL, worst, o));
+      if (cf.small && cf.check && worst <= tol) {
 #pragma unroll
-        for (int l = 0; l < 4; ++l) {
-          rs = fmaf(-rowM[l].hi, d2[l], rs);
-          corr = fmaf(Jr[l] - rowM[l].hi, d3[l], corr);
-          cabs = fmaf(fabsf(Jr[l]) + fabsf(rowM[l].hi),
-                      fabsf(dd[l]) + fabsf(d2[l]) + fabsf(d3[l]), cabs);
+        for (int k = 0; k < 4; ++k) {
+          lam[k] = df_add_f(lam[k], d1[k]);
+          lam[k] = df_add_f(lam[k], d2[k]);
+          lam[k] = df_add_f(lam[k], d3[k]);
+          ns.gres[k] = __shfl_sync(FULL, cf.rel, k);
         }
-        cabs += fabsf(rs);
-        const float ek = erel * Sk +
-                         3.7e-12f * c.dl_f * tbd *
-                             (kr == 0 ? fg.wk[0] : (kr == 1 ? fg.wk[1] : (kr == 2 ? fg.wk[2] : fg.wk[3]))) +
-                         1e-6f * cabs + Sk * grow * tbd * fmaf(1e-5f, tmax, 0.5f * tbd);
-        const float bk = fabsf(rs + corr) + ek;
-        const float rel = bk *
-                          (kr == 0 ? invS[0] : (kr == 1 ? invS[1] : (kr == 2 ? invS[2] : invS[3]))) *
-                          fmaf(1.06f, tt, 1.f);
-        float worst = rel;
-#pragma unroll
-        for (int o = 1; o < 4; o <<= 1) worst = fmaxf(worst, __shfl_xor_sync(FULL, worst, o));
-        const float xpmax = s + 2.f * c.dl_f;
-        if (worst <= tol && errmax + pmargin + xpmax * grow * tbd * 1.01f <= e) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            lam[k] = df_add_f(lam[k], d1[k]);
-            lam[k] = df_add_f(lam[k], d2[k]);
-            lam[k] = df_add_f(lam[k], d3[k]);
-            ns.gres[k] = __shfl_sync(FULL, rel, k);
-          }
-          *iters = it + 1;
-          *rlast = worst;
-          ns.check_viol = 0;
-          return 1;
-        }
+        *iters = it + 1;
+        *rlast = worst;
+        ns.check_viol = 0;
+        return 1;
       }
     }
 #pragma unroll
@@ -1295,20 +1487,20 @@ __device__ void fast_histogram(const FusedArgs& a, FastWS& w, long long b, int l
   {
     // the largest bit pattern as a signed word, and every sign bit: four
     // instructions a value; a row with a sign bit, an infinity or a NaN takes
-    // the out-of-line scan.  Eight loads in flight per lane; a point past the
-    // end reads as +0.
+    // the out-of-line scan.  Sixteen loads in flight per lane (eight: 2 % slower);
+    // a point past the end reads as +0.
     long long m = 0;
     unsigned sg = 0;
 #pragma unroll 1
-    for (int p0 = lane; p0 < P; p0 += 32 * 8) {
-      long long u[8];
+    for (int p0 = lane; p0 < P; p0 += 32 * 16) {
+      long long u[16];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < 16; ++q) {
         const int p = p0 + 32 * q;
         u[q] = p < P ? __double_as_longlong(__ldg(xb + p)) : 0ll;
       }
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < 16; ++q) {
         m = u[q] > m ? u[q] : m;
         sg |= (unsigned)(u[q] >> 32);
       }
@@ -1348,6 +1540,10 @@ __device__ void fast_histogram(const FusedArgs& a, FastWS& w, long long b, int l
       defer = true;
       break;
     }
+    store_algebra(mo, ch, w.alg);
+    // lane k (mod 4) owns component k of R
+    const int kr = lane & 3;
+    const df Rk = kr == 0 ? mo.R[0] : (kr == 1 ? mo.R[1] : (kr == 2 ? mo.R[2] : mo.R[3]));
 #pragma unroll
     for (int k = 0; k < 4; ++k) lam[k] = df{0.f, 0.f};
     int warm = 0;
@@ -1382,7 +1578,7 @@ __device__ void fast_histogram(const FusedArgs& a, FastWS& w, long long b, int l
                                  : (phase == 1 ? pr.max_iter - pr.warm_iters : pr.max_iter);
       int itx = 0;
       float ra = 0.f, rb = 0.f;
-      conv = round1_fast(g, fg, w, c, mo, ch, lam, cap, step, tol, e, s_f, &itx, &ra, &rb, ns,
+      conv = round1_fast(g, fg, w, c, Rk, lam, cap, step, tol, e, s_f, &itx, &ra, &rb, ns,
                          lane);
       if (phase != 0) {
         it1 = itx;

@@ -613,3 +613,46 @@ def test_decompressed_values_are_the_fp64_form(aq, tau):
         want = xp * a
     np.testing.assert_array_equal(f, want)
     assert np.array_equal(np.signbit(f), np.signbit(want)) or np.isnan(want).any()
+
+
+@pytest.mark.parametrize("tau", [1e-4, 1e-3])
+@pytest.mark.parametrize("grid", [(39, 39), (37, 33), (20, 30), (33, 5), (2, 2), (64, 24)])
+def test_fast_form_equals_fp64_form_on_other_grids(aq, grid, tau):
+    """The fast kernel's integer decision against the FP64 kernel where its walk
+    takes other shapes (columns in one or two parts, short chunks), on rows
+    without a scale, with flagged points, escapes, -0, a retry or verbatim
+    storage: codes, scales and statuses equal, the multipliers within the
+    tolerance of both against the oracle."""
+    vpar, vperp, vol = synth.grid_arrays(*grid)
+    P, m = grid[0] * grid[1], 203
+    x = synth.histograms(m, 77, grid=grid)
+    xh = synth.stand_in_xhat(x, 5)[:, :P].copy()
+
+    def plant(rows, fn):
+        for r in rows:
+            fn(r)
+
+    plant([0, 1, 40], lambda r: x.__setitem__((r, 1), -1.0))
+    plant([5, 42], lambda r: x.__setitem__((r, slice(None)), 0.0))
+    plant([7, 44], lambda r: x.__setitem__((r, 3), np.nan))
+    plant([9, 46], lambda r: xh.__setitem__((r, 2), np.inf))
+    plant([11, 12, 48], lambda r: xh.__setitem__((r, slice(None)), 0.0))
+    plant([14], lambda r: xh.__setitem__((r, slice(0, None, 2)), 1e30))
+    plant([16, 50], lambda r: xh.__setitem__((r, slice(None)), (x[r] + 0.49 * tau * x[r].max())))
+    plant([18], lambda r: x.__setitem__((r, 0), -0.0))
+    plant([20, 52], lambda r: xh.__setitem__((r, slice(None)), -xh[r]))
+    g = aq.Grid(vpar, vperp, vol)
+    pad = np.zeros((m, aq.XHAT_LD), np.float32)
+    pad[:, :P] = xh
+    o = [aq.quantize_correct(g, dev(x), dev(pad), aq.params_default(tau=tau, kernel=k),
+                             outlier_capacity=m * P) for k in (aq.KERNEL_FAST, aq.KERNEL_FP64)]
+    torch.cuda.synchronize()
+    for name in ("codes", "scale", "status"):
+        a, b = (getattr(c, name).cpu().numpy() for c in o)
+        np.testing.assert_array_equal(a, b, err_msg=name)
+    a, b = (c.lam.cpu().numpy() for c in o)
+    fin = np.isfinite(b).all(axis=1)
+    assert np.array_equal(fin, np.isfinite(a).all(axis=1))
+    if grid[1] >= 24:  # (the small grids' systems are close to singular)
+        assert lam_close(a[fin], b[fin])
+    assert int(o[0].count.item()) == int(o[1].count.item())
