@@ -961,27 +961,31 @@ struct ApplyArgs {
   double* f;
 };
 
-// x' = fl(xhat + c 2^k) as a double on the integer pipe; false where the
-// caller has to take the FP64 form.  The sum is an integer S (|S| < 2^53, so
-// exact) in units of the smaller of xhat's last place and 2^k, with the two at
-// most 2^37 apart.
-__device__ __forceinline__ bool level_value(int c, float xhat, int k, double* out) {
-  const unsigned v = __float_as_uint(xhat);
-  const int E = (int)((v >> 23) & 0xffu);
-  const long long m = (long long)((v & 0x7fffffu) | (E ? 0x800000u : 0u));
-  const int e = (E ? E : 1) - 150;
-  const int d = c ? k - e : 0;  // code 0: xhat itself
-  const long long S = ((long long)c << min(max(d, 0), 40)) +
-                      (((v >> 31) ? -m : m) << min(max(-d, 0), 28));
-  const unsigned long long A = S < 0 ? 0ull - (unsigned long long)S : (unsigned long long)S;
-  const int lz = __clzll((long long)A);         // >= 11
-  const int eb = e + min(d, 0) - lz + 1086;     // exponent field
-  // the leading bit of the shifted significand adds one to the exponent field
-  unsigned long long r = ((unsigned long long)(eb - 1) << 52) + (A << (lz & 63) >> 11);
-  if (S < 0) r |= 1ull << 63;
-  if (A == 0ull) r = 0ull;  // +0
+// x' = fl(xhat + c dl) as a double without the FP64 pipe, dl = 2^k a normal
+// float with room for c; false where the caller has to take the FP64 form.  The
+// sum is the pair hi + lo exactly (Knuth's two-sum, |lo| <= half a last place of
+// hi); lo in units of the double's last place, rounded half to even, is added to
+// hi's bits.  That is the rounded sum as long as it stays in hi's binade, which
+// it leaves only from a power of two downwards.
+__device__ __forceinline__ bool level_value(int c, float xhat, float dl, double* out) {
+  // float(c): 1.5 2^23 + c read off its bits
+  const float cd = __fmul_rn(__fsub_rn(__int_as_float(0x4B400000 + c), 12582912.f), dl);
+  const float hi = __fadd_rn(xhat, cd);
+  const float bb = __fsub_rn(hi, xhat);
+  const float lo = __fadd_rn(__fsub_rn(xhat, __fsub_rn(hi, bb)), __fsub_rn(cd, bb));
+  const unsigned u = __float_as_uint(hi), E = u & 0x7f800000u;
+  // 2^52 / 2^floor(log2 |hi|) with hi's sign
+  const float sc = __uint_as_float((0x99000000u - E) ^ (u & 0x80000000u));
+  const float t = __fmul_rn(lo, sc);  // |t| <= 2^28
+  // round to nearest even in two steps of twelve and seventeen bits
+  const float ma = fmaf(t, 1.f / 4096.f, 12582912.f);
+  const float mb = __fadd_rn(fmaf(__fsub_rn(ma, 12582912.f), -4096.f, t), 12582912.f);
+  const int n = (__float_as_int(ma) - 0x4B400000) * 4096 + (__float_as_int(mb) - 0x4B400000);
+  const unsigned hw = (((u << 1) >> 4) + 0x38000000u) | (u & 0x80000000u);
+  const unsigned long long r =
+      (((unsigned long long)hw << 32) | (u << 29)) + (unsigned long long)(long long)n;
   *out = __longlong_as_double((long long)r);
-  return E != 255 && d <= 37 && d >= -28 && eb >= 2 && eb <= 2045;
+  return E - (52u << 23) <= (202u << 23) && ((u << 9) != 0u || t >= 0.f);
 }
 
 // the same in FP64; a call, since inline it would be computed for every point
@@ -990,18 +994,62 @@ __device__ __noinline__ double level_value_fp64(int c, float xhat, double dl) {
   return __dadd_rn((double)xhat, __dmul_rn((double)c, dl));
 }
 
-// One warp per histogram, four points of a lane in flight.  The FP64 form of
-// a point is six instructions of the FP64 pipe (two conversions, the product
-// with the bin width, the sum and the two factors), 4,600 cycles of an SM per
-// histogram.  Here x' is put together on the integer pipe with the same bits
-// and the two factors are the FP64 pipe's only work per point: 150,001
-// histograms 4,060 -> 1,224 us.  (The first factor on the integer pipe too:
-// 164 instructions a point, 1,545 us.)
+// One column segment of a histogram: rows [j0, j1) of column i.  One point a
+// turn, its operands loaded a row ahead.
+__device__ __forceinline__ void apply_column(int i, int j0, int j1, int n_par, const int16_t* cb,
+                                             const float* xb, double* fb, const double* ta,
+                                             const double* tb, float dl_f, double dl) {
+  if (j0 >= j1) return;
+  const double ai = ta[i];
+  int p = j0 * n_par + i;
+  int cn = __ldg(cb + p);
+  float hn = __ldg(xb + p);
+#pragma unroll 1
+  for (int j = j0; j < j1; ++j) {
+    const int c = cn;
+    const float xh = hn;
+    const int q = p;
+    p += n_par;
+    if (j + 1 < j1) {
+      cn = __ldg(cb + p);
+      hn = __ldg(xb + p);
+    }
+    if (c == AEQC_CODE_ESCAPE) continue;  // scatter_corrected_kernel writes it
+    double x;
+    if (c == AEQC_CODE_ZERO) x = 0.0;
+    else if (!level_value(c, xh, dl_f, &x)) x = level_value_fp64(c, xh, dl);
+    fb[q] = corr_kl(x, ai, tb[j]);
+  }
+}
+
+// One warp per histogram.  The FP64 form of a point is six instructions of the
+// FP64 pipe (two conversions, the product with the bin width, the sum and the
+// two factors), 4,600 cycles of an SM per histogram.  Here x' is put together on
+// the FP32 and integer pipes with the same bits and the two factors are the FP64
+// pipe's only work per point, 1,500 cycles, which bounds the kernel.  Each lane
+// walks down columns, so that its factor in v_par stays in a register and the
+// loop is short: a body that outgrows the instruction buffers costs more than
+// its instructions (four points a turn with a 64-bit integer sum: 1,224 us for
+// 150,001 histograms; this form 1,090 us, the FP64 pipe 78 % busy; the FP64
+// form 4,060 us).
 __global__ void __launch_bounds__(128, 10) apply_kernel(const __grid_constant__ ApplyArgs a) {
   __shared__ double ta[4][AEQC_MAX_NPAR], tb[4][AEQC_MAX_NPERP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const GridK& g = a.g;
   const long long nw = (long long)gridDim.x * 4;
+  // lane's columns: column `lane` of the first 32 (where there are as many), and
+  // a chunk of rows of one of the rw others
+  const int cw = g.n_par >= 32 ? 32 : 0, rw = g.n_par - cw;
+  int c2 = 0, k0 = 0, k1 = 0;
+  if (rw) {
+    const int nchunk = 32 / rw, rpc = (g.n_perp + nchunk - 1) / nchunk;
+    if (lane < rw * nchunk) {
+      const int chunk = lane / rw;
+      c2 = cw + lane - chunk * rw;
+      k0 = chunk * rpc;
+      k1 = min(g.n_perp, k0 + rpc);
+    }
+  }
   for (long long b = (long long)blockIdx.x * 4 + warp; b < a.n; b += nw) {
     const unsigned st = a.status[b];
     double lam[4];
@@ -1018,39 +1066,26 @@ __global__ void __launch_bounds__(128, 10) apply_kernel(const __grid_constant__ 
                           : bin_width(a.prm.tau, a.scale[b],
                                       (st & AEQC_ST_ALPHA_RETRY) ? a.prm.alpha4 : a.prm.alpha);
     const int de = (int)((unsigned long long)__double_as_longlong(dl) >> 52);
-    // the integer form: a normal bin width 2^k
-    const bool fast = a.prm.loss == 0 && de >= 1 && de <= 2046;
-    const int k = de - 1023;
     const int16_t* cb = a.codes + b * g.P;
     const float* xb = a.xhat + b * a.ld;
     double* fb = a.f + b * g.P;
-    PointIter pi(lane, g.n_par);
-    while (pi.p < g.P) {
-      int c[4];
-      float xh[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int p = pi.p + 32 * q;
-        c[q] = p < g.P ? __ldg(cb + p) : 0;
-        xh[q] = p < g.P ? __ldg(xb + p) : 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q, pi.next()) {
-        if (pi.p >= g.P || (c[q] == AEQC_CODE_ESCAPE && !zero)) continue;
-        double f;
-        if (fast) {
-          const bool empty = c[q] == AEQC_CODE_ZERO;
-          if (!level_value(empty ? 0 : c[q], empty ? 0.f : xh[q], k, &f) && !empty)
-            f = level_value_fp64(c[q], xh[q], dl);
-          f = corr_kl(f, ta[warp][pi.i], tb[warp][pi.j]);
-        } else {
-          const double xp = zero || c[q] == AEQC_CODE_ZERO
-                                ? 0.0
-                                : __dadd_rn((double)xh[q], __dmul_rn((double)c[q], dl));
-          f = a.prm.loss == 0 ? corr_kl(xp, ta[warp][pi.i], tb[warp][pi.j])
-                              : corr_l2(xp, lam, g.vpar[pi.i], g.vperp2[pi.j]);
-        }
-        fb[pi.p] = f;
+    // the float form: dl = 2^k and c dl normal floats (a bin width is a power of
+    // two or no normal number)
+    if (a.prm.loss == 0 && de >= 1023 - 126 && de <= 1023 + 100) {
+      const float dl_f = __int_as_float((de - 1023 + 127) << 23);
+#pragma unroll 1
+      for (int part = cw ? 0 : 1; part < 2; ++part)
+        apply_column(part ? c2 : lane, part ? k0 : 0, part ? k1 : g.n_perp, g.n_par, cb, xb, fb,
+                     ta[warp], tb[warp], dl_f, dl);
+    } else {
+      PointIter pi(lane, g.n_par);
+#pragma unroll 1
+      for (; pi.p < g.P; pi.next()) {
+        const int c = __ldg(cb + pi.p);
+        if (c == AEQC_CODE_ESCAPE && !zero) continue;
+        const double xp = zero || c == AEQC_CODE_ZERO ? 0.0 : level_value_fp64(c, __ldg(xb + pi.p), dl);
+        fb[pi.p] = a.prm.loss == 0 ? corr_kl(xp, ta[warp][pi.i], tb[warp][pi.j])
+                                   : corr_l2(xp, lam, g.vpar[pi.i], g.vperp2[pi.j]);
       }
     }
     __syncwarp();
