@@ -42,6 +42,26 @@ __device__ __forceinline__ bool tile_of(const GemmArgs& a, long long t, int* g, 
   return true;
 }
 
+// one output from its sum (rs: the row's scale or its inverse, bb: its bias)
+__device__ __forceinline__ void write_one(const GemmArgs& a, float v, float* dst, float rs,
+                                          float bb) {
+  switch (a.epi) {
+    case EPI_PLAIN:
+      v = a.beta != 0.f ? fmaf(a.alpha, v, a.beta * *dst) : a.alpha * v;
+      break;
+    case EPI_BIAS_ACT:
+      v = act_apply(a.act, v + bb);
+      break;
+    case EPI_ROWSCALE_BIAS_ACT:
+      v = act_apply(a.act, fmaf(v, rs, bb));
+      break;
+    default:  // EPI_DENORM
+      v = rs * (v + bb);
+      break;
+  }
+  *dst = v;
+}
+
 template <bool A_F64>
 __global__ void __launch_bounds__(NT, 2) gemm_kernel(const GemmArgs a) {
   __shared__ __align__(16) float As[2][BK][BM];
@@ -179,25 +199,118 @@ __global__ void __launch_bounds__(NT, 2) gemm_kernel(const GemmArgs a) {
       const int c = (j < 4) ? tx * 4 + j : 64 + tx * 4 + (j - 4);
       const int gc = n0 + c;
       if (gc >= a.N) continue;
-      float v = acc[i][j];
-      float* dst = a.C + gr * a.ldc + gc;
-      const float bb = bias ? bias[gc] : 0.f;
-      switch (a.epi) {
-        case EPI_PLAIN:
-          v = a.beta != 0.f ? fmaf(a.alpha, v, a.beta * *dst) : a.alpha * v;
-          break;
-        case EPI_BIAS_ACT:
-          v = act_apply(a.act, v + bb);
-          break;
-        case EPI_ROWSCALE_BIAS_ACT:
-          v = act_apply(a.act, fmaf(v, rs, bb));
-          break;
-        default:  // EPI_DENORM
-          v = rs * (v + bb);
-          break;
-      }
-      *dst = v;
+      write_one(a, acc[i][j], a.C + gr * a.ldc + gc, rs, bias ? bias[gc] : 0.f);
     }
+  }
+}
+
+// The same product where 128 x 128 tiles are too few to fill the GPU: 16 x 32
+// tiles, two outputs a thread, K in chunks of 64 with the next chunk's loads in
+// flight.  One CTA of the other form does 64 x 128 outputs with K = 1521 in 191
+// steps, each waiting for its loads: 363 us (FP64 A), and 12 CTAs of 128 columns
+// with K = 128 26 us; this form 40 and 7 us.  Every output is the same sum in
+// the same order: identical bits.
+constexpr int SM_ = 16, SN_ = 32, SK_ = 64;
+
+template <bool A_F64>
+__global__ void __launch_bounds__(256) gemm_small_kernel(const GemmArgs a) {
+  __shared__ float As[2][SK_][SM_ + 1];
+  __shared__ float Bs[2][SK_][SN_ + 1];
+  __shared__ unsigned long long rowmax_s[SM_];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const long long r0 = (long long)blockIdx.y * SM_;
+  const int n0 = blockIdx.x * SN_;
+  const bool a_kc = A_F64 || a.sak == 1, b_kc = a.sbk == 1;
+  if (tid < SM_) rowmax_s[tid] = 0ull;
+  // element e of the thread: consecutive threads on consecutive k where the
+  // operand is contiguous in k, else on consecutive rows (columns)
+  auto a_row = [&](int e) { return a_kc ? (tid >> 6) + 4 * e : tid & 15; };
+  auto a_k = [&](int e) { return a_kc ? tid & 63 : (tid >> 4) + 16 * e; };
+  auto b_col = [&](int e) { return b_kc ? (tid >> 6) + 4 * e : lane; };
+  auto b_k = [&](int e) { return b_kc ? tid & 63 : warp + 8 * e; };
+  double ad[4];
+  float ra[4], rb[8];
+  // largest value of the thread's rows as bits: zero, finite or infinite values
+  // only (max(x) semantics: NaN and negatives never win)
+  long long rmax[4] = {0, 0, 0, 0};
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const long long gr = r0 + a_row(e);
+      const int gk = k0 + a_k(e);
+      const bool in = gr < a.M && gk < a.K;
+      const long long at = gr * a.sam + (long long)gk * a.sak;
+      if (A_F64) ad[e] = in ? __ldg(static_cast<const double*>(a.A) + at) : 0.0;
+      else ra[e] = in ? __ldg(static_cast<const float*>(a.A) + at) : 0.f;
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int gc = n0 + b_col(e), gk = k0 + b_k(e);
+      rb[e] = gc < a.N && gk < a.K
+                  ? __ldg(a.B + (long long)gk * a.sbk + (long long)gc * a.sbn)
+                  : 0.f;
+    }
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (A_F64) {
+        const long long u = __double_as_longlong(ad[e]);
+        if (u > rmax[e] && u <= 0x7FF0000000000000ll) rmax[e] = u;
+        ra[e] = (float)ad[e];
+      }
+      As[buf][a_k(e)][a_row(e)] = ra[e];
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) Bs[buf][b_k(e)][b_col(e)] = rb[e];
+  };
+  // both forms pad K to whole steps of BK with zeros
+  const int Kp = (a.K + BK - 1) / BK * BK;
+  float acc0 = 0.f, acc1 = 0.f;
+  load(0);
+  store(0);
+  __syncthreads();
+  for (int k0 = 0, buf = 0; k0 < Kp; k0 += SK_, buf ^= 1) {
+    const bool more = k0 + SK_ < Kp;
+    if (more) load(k0 + SK_);
+    const int kn = min(SK_, Kp - k0);
+#pragma unroll 8
+    for (int k = 0; k < kn; ++k) {
+      const float b = Bs[buf][k][lane];
+      acc0 = fmaf(As[buf][k][2 * warp], b, acc0);
+      acc1 = fmaf(As[buf][k][2 * warp + 1], b, acc1);
+    }
+    if (more) store(buf ^ 1);
+    __syncthreads();
+  }
+  if (A_F64) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      long long m = rmax[e];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long v = __shfl_xor_sync(0xffffffffu, m, o);
+        m = v > m ? v : m;
+      }
+      if (lane == 0) atomicMax(&rowmax_s[a_row(e)], (unsigned long long)m);
+    }
+    __syncthreads();
+    if (tid < SM_ && a.scale_out && blockIdx.x == 0 && r0 + tid < a.M)
+      a.scale_out[r0 + tid] = __longlong_as_double((long long)rowmax_s[tid]);
+  }
+  const int gc = n0 + lane;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int r = 2 * warp + i;
+    const long long gr = r0 + r;
+    if (gr >= a.M || gc >= a.N) continue;
+    float rs = 1.f;
+    if (a.epi == EPI_DENORM) rs = (float)a.scale_in[gr];
+    if (A_F64) {
+      const double s = __longlong_as_double((long long)rowmax_s[r]);
+      rs = (s > 0.0 && isfinite(s)) ? (float)(1.0 / s) : 0.f;
+    }
+    write_one(a, i ? acc1 : acc0, a.C + gr * a.ldc + gc, rs, a.bias ? a.bias[gc] : 0.f);
   }
 }
 
@@ -338,6 +451,8 @@ __global__ void __launch_bounds__(256) bias_act_tiny_kernel(const GemmArgs a) {
   }
 }
 
+constexpr long long SMALL_MAX_TILES = 76;
+
 int launch_gemm(const GemmArgs& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0) return AEQC_OK;
   if (!a.a_f64 && a.epi == EPI_BIAS_ACT && a.N <= 8 && a.K <= 8 && a.sak == 1 &&
@@ -361,6 +476,16 @@ int launch_gemm(const GemmArgs& a, cudaStream_t s) {
   if (tiles > 2147483647LL || tiles > 65535LL * 65535LL)
     return set_error(AEQC_EUNSUPPORTED, "gemm: too many row tiles");
   dim3 grid((a.N + BN - 1) / BN, (unsigned)tiles);
+  // up to half the SMs' worth of 128 x 128 tiles: 32 times as many small ones (a
+  // tile of the large form then waits alone on its SM for every load).  Encoding
+  // with H = 128: 10 rows 344 -> 69 us, 1,000 rows (8 tiles) 379 -> 87, 9,000
+  // rows (71 tiles) 454 -> 380 us.
+  if (a.n_groups <= 1 && tiles * grid.x <= SMALL_MAX_TILES) {
+    dim3 gs((a.N + SN_ - 1) / SN_, (unsigned)((a.M + SM_ - 1) / SM_));
+    if (a.a_f64) gemm_small_kernel<true><<<gs, 256, 0, s>>>(a);
+    else gemm_small_kernel<false><<<gs, 256, 0, s>>>(a);
+    return check_launch("gemm_small_kernel");
+  }
   if (tiles > 65535) {
     // grid.y is limited to 65535: split into several launches over row ranges
     GemmArgs b = a;

@@ -375,3 +375,24 @@ def test_float32_multipliers_against_oracle(aq, trained):
     assert e64 <= 1e-11
     assert e32 <= 1e-6
     print("moment error with float64 / float32 multipliers: %.2e / %.2e" % (e64, e32))
+
+
+@pytest.mark.parametrize("n", [1, 15, 17, 64, 130, 1000])
+@pytest.mark.parametrize("H,L", [(128, 16), (96, 8)])
+def test_small_batches_take_the_same_sums(aq, n, H, L):
+    """Products with few 128 x 128 tiles run on 16 x 32 tiles: every row's scale,
+    latent and decoded values have the bits they have inside a large batch (a
+    container written with one is read back with the other)."""
+    P, N = synth.P, 128 * 77 + 5
+    m, _ = make_model(aq, P, H, L, True, 1, 1, 11)
+    x = synth.histograms(n, 21)
+    if n > 15:
+        x[3, 7], x[5, 9], x[6] = np.nan, np.inf, -x[6]
+    big = dev(np.tile(x, (N // n + 1, 1))[:N])
+    z1, s1 = aq.ae_encode(m, dev(x))
+    z2, s2 = aq.ae_encode(m, big)
+    h1 = aq.ae_decode(m, z1, s1)[:, :P]
+    h2 = aq.ae_decode(m, z2, s2)[:, :P]
+    torch.cuda.synchronize()
+    for a, b in ((z1, z2), (s1, s2), (h1, h2)):
+        np.testing.assert_array_equal(a.cpu().numpy(), b[:n].cpu().numpy())
