@@ -752,7 +752,11 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(CT, 3)
   __shared__ ClusterShared sh;
   const unsigned rank = cluster_rank();
   const int cnt = all ? all : *count;
-  if (cnt > most) return;
+  if (cnt > most) return;  // the same in every block
+  // A block's shared memory may be written by another one only once it is known
+  // to have started, which a barrier of the cluster shows and nothing else does
+  // (process_cluster writes into all eight blocks before its first barrier).
+  cluster_sync();
   int turn = 0;
   const int nc = gridDim.x / CL;
   if (all && blockIdx.x == 0 && threadIdx.x == 0) *count = all;
