@@ -1752,12 +1752,14 @@ int make_fast_grid(const GridK& g, FastGridK* out) {
   f.vmax = (float)vmax;
   f.wmax = (float)g.vperp2[g.n_perp - 1];
   {
-    const int rw = g.n_par - (g.n_par >= 32 ? 32 : 0);  // >= 1 (n_par in [2, 64])
-    f.seg_nchunk = 32 / rw;
-    f.seg_rpc = (g.n_perp + f.seg_nchunk - 1) / f.seg_nchunk;
-    f.seg_mul = (65536 + rw - 1) / rw;
-    for (int l = 0; l < 32; ++l)
-      if ((l * f.seg_mul) >> 16 != l / rw) return AEQC_OK;  // never: 2^16 > 32 rw
+    const int rw = g.n_par - (g.n_par >= 32 ? 32 : 0);  // 0 for 32 columns: no second part
+    if (rw) {
+      f.seg_nchunk = 32 / rw;
+      f.seg_rpc = (g.n_perp + f.seg_nchunk - 1) / f.seg_nchunk;
+      f.seg_mul = (65536 + rw - 1) / rw;
+      for (int l = 0; l < 32; ++l)
+        if ((l * f.seg_mul) >> 16 != l / rw) return AEQC_OK;  // never: 2^16 > 32 rw
+    }
   }
   *out = f;
   return AEQC_OK;
