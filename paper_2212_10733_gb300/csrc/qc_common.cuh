@@ -105,7 +105,8 @@ __device__ __forceinline__ int quant_point_fp64(double x, double xh, double dl, 
 }
 
 // Solve M d = r, M symmetric positive definite (upper triangle given as the
-// 10 entries m00 m01 m02 m03 m11 m12 m13 m22 m23 m33), by Cholesky.
+// 10 entries m00 m01 m02 m03 m11 m12 m13 m22 m23 m33), by Cholesky, every
+// rounding written out (the cluster form takes the same steps, a row a lane).
 // Returns 0 on success, -1 when a pivot is not positive or d is not finite.
 __device__ __forceinline__ int chol_solve4(const double m[10], const double r[4], double d[4]) {
   double a[4][4];
@@ -127,12 +128,12 @@ __device__ __forceinline__ int chol_solve4(const double m[10], const double r[4]
     for (int l = 0; l <= k; ++l) {
       double s = a[k][l];
 #pragma unroll
-      for (int q = 0; q < l; ++q) s -= L[k][q] * L[l][q];
+      for (int q = 0; q < l; ++q) s = __fma_rn(-L[k][q], L[l][q], s);
       if (k == l) {
         if (!(s > 0.0)) return -1;
-        L[k][k] = sqrt(s);
+        L[k][k] = __dsqrt_rn(s);
       } else {
-        L[k][l] = s / L[l][l];
+        L[k][l] = __ddiv_rn(s, L[l][l]);
       }
     }
   }
@@ -141,15 +142,15 @@ __device__ __forceinline__ int chol_solve4(const double m[10], const double r[4]
   for (int k = 0; k < 4; ++k) {
     double s = r[k];
 #pragma unroll
-    for (int q = 0; q < k; ++q) s -= L[k][q] * y[q];
-    y[k] = s / L[k][k];
+    for (int q = 0; q < k; ++q) s = __fma_rn(-L[k][q], y[q], s);
+    y[k] = __ddiv_rn(s, L[k][k]);
   }
 #pragma unroll
   for (int k = 3; k >= 0; --k) {
     double s = y[k];
 #pragma unroll
-    for (int q = k + 1; q < 4; ++q) s -= L[q][k] * d[q];
-    d[k] = s / L[k][k];
+    for (int q = k + 1; q < 4; ++q) s = __fma_rn(-L[q][k], d[q], s);
+    d[k] = __ddiv_rn(s, L[k][k]);
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k)

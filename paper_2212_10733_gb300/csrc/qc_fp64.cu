@@ -32,23 +32,47 @@ __device__ __forceinline__ double vol_of(const GridK& g, int p) {
   return g.has_vol ? __ldg(g.vol + p) : g.vol_uniform;
 }
 
+// One point's share of the sums, with every rounding written out: the cluster
+// form further below forms the same sums from the same terms in the same order
+// and has to get the same bits (left to contraction, the compiler decides per
+// kernel which products it fuses).
+struct Products {
+  double v, w, vv, vvv;  // y v, y v_perp^2, y v^2, y v^3
+};
+__device__ __forceinline__ Products products_of(double y, double v, double v2) {
+  Products t;
+  t.v = __dmul_rn(y, v);
+  t.w = __dmul_rn(y, v2);
+  t.vv = __dmul_rn(t.v, v);
+  t.vvv = __dmul_rn(t.vv, v);
+  return t;
+}
+__device__ __forceinline__ void add_moments(double y, double v, double v2, double& a0, double& a1,
+                                            double& a2, double& a3) {
+  const double yv = __dmul_rn(y, v);
+  a0 = __dadd_rn(a0, y);
+  a1 = __dadd_rn(a1, yv);
+  a2 = __fma_rn(y, v2, a2);
+  a3 = __fma_rn(yv, v, a3);
+}
+__device__ __forceinline__ void add_abs_moments(double y, double v, double v2, double& s0,
+                                                double& s1, double& s2, double& s3) {
+  s0 = __dadd_rn(s0, y);
+  s1 = __fma_rn(y, fabs(v), s1);
+  s2 = __fma_rn(y, v2, s2);
+  s3 = __fma_rn(__dmul_rn(y, v), v, s3);
+}
+
 // Q_k(x) and S_k(x) = sum vol |phi_k| |x| for the histogram in xs.
 __device__ void moments_warp(const GridK& g, const double* xs, double Q[4], double S[4],
                              int lane) {
   double q0 = 0, q1 = 0, q2 = 0, q3 = 0, s0 = 0, s1 = 0, s2 = 0, s3 = 0;
   PointIter it(lane, g.n_par);
   for (; it.p < g.P; it.next()) {
-    double v = g.vpar[it.i], v2 = g.vperp2[it.j];
-    double w = vol_of(g, it.p) * xs[it.p];
-    double aw = fabs(w);
-    q0 += w;
-    q1 += w * v;
-    q2 += w * v2;
-    q3 += w * v * v;
-    s0 += aw;
-    s1 += aw * fabs(v);
-    s2 += aw * v2;
-    s3 += aw * v * v;
+    const double v = g.vpar[it.i], v2 = g.vperp2[it.j];
+    const double w = __dmul_rn(vol_of(g, it.p), xs[it.p]);
+    add_moments(w, v, v2, q0, q1, q2, q3);
+    add_abs_moments(fabs(w), v, v2, s0, s1, s2, s3);
   }
   Q[0] = wsum(q0); Q[1] = wsum(q1); Q[2] = wsum(q2); Q[3] = wsum(q3);
   S[0] = wsum(s0); S[1] = wsum(s1); S[2] = wsum(s2); S[3] = wsum(s3);
@@ -79,31 +103,25 @@ __device__ void eval_warp(const GridK& g, WS& w, const double lam[4], const doub
     double f, wm;
     if (loss == 0) {
       f = corr_kl(w.xp[it.p], w.ta[it.i], w.tb[it.j]);
-      wm = f * vol;
+      wm = __dmul_rn(f, vol);
     } else {
       f = corr_l2(w.xp[it.p], lam, v, v2);
       wm = vol;
     }
-    double fv = f * vol, af = fabs(fv);
-    a0 += fv;
-    a1 += fv * v;
-    a2 += fv * v2;
-    a3 += fv * v * v;
-    s0 += af;
-    s1 += af * fabs(v);
-    s2 += af * v2;
-    s3 += af * v * v;
+    const double fv = __dmul_rn(f, vol);
+    add_moments(fv, v, v2, a0, a1, a2, a3);
+    add_abs_moments(fabs(fv), v, v2, s0, s1, s2, s3);
     if (want_M) {
-      double wv = wm * v;
-      m00 += wm;
-      m01 += wv;
-      m02 += wm * v2;
-      m03 += wv * v;
-      m12 += wv * v2;
-      m13 += wv * v * v;
-      m22 += wm * v2 * v2;
-      m23 += wv * v * v2;
-      m33 += wv * v * v * v;
+      const Products t = products_of(wm, v, v2);
+      m00 = __dadd_rn(m00, wm);
+      m01 = __dadd_rn(m01, t.v);
+      m02 = __dadd_rn(m02, t.w);
+      m03 = __dadd_rn(m03, t.vv);
+      m12 = __fma_rn(t.v, v2, m12);
+      m13 = __dadd_rn(m13, t.vvv);
+      m22 = __fma_rn(t.w, v2, m22);
+      m23 = __fma_rn(t.vv, v2, m23);
+      m33 = __fma_rn(t.vvv, v, m33);
     }
   }
   r.A[0] = wsum(a0); r.A[1] = wsum(a1); r.A[2] = wsum(a2); r.A[3] = wsum(a3);
@@ -137,7 +155,7 @@ __device__ int round1_warp(const GridK& g, WS& w, const double Q[4], double lam[
     for (int k = 0; k < 4; ++k) gk[k] = e.A[k] - Q[k];
     if (chol_solve4(e.M, gk, d) != 0) return 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) lam[k] += step * d[k];
+    for (int k = 0; k < 4; ++k) lam[k] = __fma_rn(step, d[k], lam[k]);
   }
 }
 
@@ -422,30 +440,39 @@ __global__ void __launch_bounds__(WPC * 32) fused_fp64_list_kernel(const FusedAr
 // of an SM issues one in 64 cycles: 0.67 ms, whatever else the chip does.  The
 // fast kernel defers a handful of histograms in a hundred thousand, and a
 // small batch has fewer histograms than the chip has SMs, so here a cluster of
-// CL blocks (24 quarter SMs at work) takes one histogram, a thread per point.  Sums
-// go through the warp (reduce-scatter), the block and the cluster's shared
-// memory; every block forms the same totals in the same order, and its first
-// warp takes the same decisions.  Only the ordinary course is handled: a
-// histogram with non-finite, negative or no input, one that round 1 does not
-// solve, warm starts, features, volumes per cell and the L2 loss are left to
-// the warp kernels.  13 deferred histograms: 675 -> 67 us; 64 histograms in
-// the FP64 form: 722 -> 111 us.
+// CL blocks takes one histogram, a thread per point.  The sums are those of
+// the warp form to the bit, so that a histogram's result does not depend on
+// how many others its call has: each of the twelve different sums belongs to
+// one warp, whose lane l adds the terms of the points l, l + 32, ... in that
+// order; the terms come from the blocks of the points through the cluster's
+// shared memory, every block summing one kind of term.  The last block solves
+// for the step (chol_solve4's operations, a row of the matrix a lane) and
+// sends it to the others.  Only the ordinary course is handled: a histogram
+// with non-finite, negative or no input, one that round 1 does not solve, warm
+// starts, features, volumes per cell and the L2 loss are left to the warp
+// kernels.  What bounds it is the latency of a step: three cluster barriers,
+// 48 dependent additions, and the solution's square roots and divisions.  FP64
+// form of n histograms of 39 x 39 (tau = 1e-3), a cluster / a warp each: n = 1
+// 66 / 348 us, 16 80 / 445, 64 145 / 731, 128 218 / 730, 320 497 / 731 us.
 constexpr int CL = 8;
 constexpr int CT = AEQC_MAX_P / CL;  // threads of a block: a point each
 constexpr int CWARPS = CT / 32;
-constexpr int CV = 16;               // values of one exchange
-static_assert(CT % 32 == 0, "whole warps");
+constexpr unsigned SOLVER = CL - 1;
+static_assert(CT % 32 == 0 && CT >= AEQC_MAX_NPAR && CL * CWARPS <= 64, "block shape");
+
+// A_k (= S_k but for k = 1), S_1 and the entries of M that are no A_k (M11 = M03)
+enum Sum { A0, A1, A2, A3, S1, M02, M03, M12, M13, M22, M23, M33, SUMS };
+enum Weight { ONE, V, ABSV, W };
 
 struct ClusterShared {
-  double part[CWARPS][CV];     // this block's warps
-  double all[2][CL][CV];       // the blocks' totals, alternating between exchanges
-  unsigned long long umax[CL * CWARPS];
-  int bad[CL * CWARPS];
-  int esc[CL * CWARPS];
-  long long base;
+  double val[AEQC_MAX_P];  // the terms that this block sums
+  double v[AEQC_MAX_NPAR], av[AEQC_MAX_NPAR], w[AEQC_MAX_NPERP];  // v, |v|, v_perp^2
   double ta[AEQC_MAX_NPAR], tb[AEQC_MAX_NPERP];
+  unsigned long long umax[CL * CWARPS];
+  unsigned flags[CL * CWARPS];
+  long long base;
   double lam[4];
-  double tot[CV];
+  double tot[SUMS], Q[4], S1;  // block SOLVER only
   int verdict;
 };
 
@@ -469,122 +496,93 @@ __device__ __forceinline__ unsigned remote(const void* p, unsigned r) {
 __device__ __forceinline__ void put_u64(const void* p, unsigned r, unsigned long long v) {
   asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(remote(p, r)), "l"(v) : "memory");
 }
+__device__ __forceinline__ void put_f64(const double* p, unsigned r, double v) {
+  put_u64(p, r, (unsigned long long)__double_as_longlong(v));
+}
 __device__ __forceinline__ void put_u32(const void* p, unsigned r, unsigned v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(p, r)), "r"(v) : "memory");
 }
 
-// Totals of v[0 .. CV) over the cluster, to sh.tot in every block (fixed order).
-__device__ __forceinline__ void cluster_sums(ClusterShared& sh, double (&v)[CV], int& turn,
-                                             unsigned rank) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16, n = 8; n >= 1; o >>= 1, n >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < n; ++i) {
-      const double send = up ? v[i] : v[n + i];
-      const double keep = up ? v[n + i] : v[i];
-      v[i] = keep + __shfl_xor_sync(FULL, send, o);
-    }
+__device__ __forceinline__ void load_weights(const GridK& g, ClusterShared& sh) {
+  const int t = threadIdx.x;
+  if (t < g.n_par) {
+    sh.v[t] = g.vpar[t];
+    sh.av[t] = fabs(g.vpar[t]);
   }
-  const double mine = v[0] + __shfl_xor_sync(FULL, v[0], 1);
-  if (!(lane & 1)) sh.part[warp][lane >> 1] = mine;  // lane bits 4..1 are the value's index
-  __syncthreads();
-  double(&all)[CL][CV] = sh.all[turn & 1];
-  ++turn;
-  if (warp == 0) {
-    const int idx = lane & (CV - 1), half = lane >> 4;
-    double t = sh.part[half * (CWARPS / 2)][idx];
-#pragma unroll
-    for (int w = 1; w < CWARPS / 2; ++w) t += sh.part[half * (CWARPS / 2) + w][idx];
-    t += __shfl_xor_sync(FULL, t, 16);
-    // each half-warp sends to half of the blocks
-    for (unsigned r = half * (CL / 2); r < (half + 1) * (CL / 2); ++r)
-      put_u64(&all[rank][idx], r, (unsigned long long)__double_as_longlong(t));
-  }
-  cluster_sync();
-  if (warp == 0) {
-    const int idx = lane & (CV - 1), half = lane >> 4;
-    double t = all[half * (CL / 2)][idx];
-#pragma unroll
-    for (int r = 1; r < CL / 2; ++r) t += all[half * (CL / 2) + r][idx];
-    t += __shfl_xor_sync(FULL, t, 16);
-    if (half == 0) sh.tot[idx] = t;
-    __syncwarp();
+  if (t < g.n_perp) sh.w[t] = g.vperp2[t];
+}
+
+// The terms of point p (y = vol f) to the blocks that sum them
+template <bool MATRIX>
+__device__ __forceinline__ void send_terms(const ClusterShared& sh, int p, double y, double v,
+                                           double v2) {
+  const Products t = products_of(y, v, v2);
+  put_f64(&sh.val[p], 0, y);
+  put_f64(&sh.val[p], 1, y);
+  put_f64(&sh.val[p], 2, t.v);
+  if (MATRIX) {
+    put_f64(&sh.val[p], 3, t.v);
+    put_f64(&sh.val[p], 4, t.w);
+    put_f64(&sh.val[p], 5, t.vv);
+    put_f64(&sh.val[p], 6, t.vvv);
   }
 }
 
-// M d = r (chol_solve4's arguments): FP32 Cholesky of the unit-diagonal scaling
-// and one FP64 refinement, which leaves an error of about (6e-8 cond)^2; a
-// pivot below 1e-3 takes the FP64 factorisation (its square roots and
-// divisions are some 400 FP64 instructions on one warp).
-__device__ __forceinline__ int solve4(const double m[10], const double r[4], double d[4]) {
-  const int ix[4][4] = {{0, 1, 2, 3}, {1, 4, 5, 6}, {2, 5, 7, 8}, {3, 6, 8, 9}};
-  float sc[4], L[4][4], inv[4];
-  bool ok = true;
+// sums of blocks 0 .. 6 (a warp each) and the weights of their terms
+__constant__ signed char SUM_OF[2][CL] = {{A0, S1, A1, M12, M02, M03, M13, -1},
+                                          {A2, -1, A3, -1, M22, M23, M33, -1}};
+__constant__ signed char WEIGHT_OF[2][CL] = {{ONE, ABSV, ONE, W, ONE, ONE, ONE, ONE},
+                                             {W, ONE, V, ONE, W, W, V, ONE}};
+
+// The sums (those up to `last`) of the terms sent before, to block SOLVER.  With the
+// weight one the fused product is the plain sum.
+__device__ __forceinline__ void sum_terms(const GridK& g, ClusterShared& sh, unsigned rank,
+                                          int last) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  cluster_sync();
+  const int sum = warp < 2 ? SUM_OF[warp][rank] : -1;
+  if (sum >= 0 && sum <= last) {
+    const int wt = WEIGHT_OF[warp][rank];
+    const double* tab = wt == W ? sh.w : (wt == V ? sh.v : sh.av);
+    double acc = 0.0;
+    PointIter it(lane, g.n_par);
+#pragma unroll 4
+    for (; it.p < g.P; it.next())
+      acc = __fma_rn(sh.val[it.p], wt == ONE ? 1.0 : tab[wt == W ? it.j : it.i], acc);
+    acc = wsum(acc);
+    if (lane == 0) put_f64(&sh.tot[sum], SOLVER, acc);
+  }
+  cluster_sync();
+}
+
+// chol_solve4 for the matrix of sh.tot with a row a lane: lanes 0 to 3 hold the
+// rows of L, lane 4 the forward solution of the right-hand side (lane k's gk is
+// its component k), which the same operations produce.  All lanes return d.
+__device__ __forceinline__ int solve_rows(const ClusterShared& sh, double gk, double (&d)[4],
+                                          int lane) {
+  const int ix[4][4] = {{A0, A1, M02, M03}, {A1, M03, M12, M13}, {M02, M12, M22, M23},
+                        {M03, M13, M23, M33}};
+  double L[4], diag[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float t = (float)m[ix[k][k]];
-    ok = ok && t > 1e-30f && t < 1e30f;
-    sc[k] = ok ? rsqrtf(t) : 0.f;
+  for (int l = 0; l < 4; ++l) {
+    const double rhs = __shfl_sync(FULL, gk, l);
+    double t = sh.tot[lane == 0 ? ix[0][l] : (lane == 1 ? ix[1][l] : (lane == 2 ? ix[2][l]
+                                                                                : ix[3][l]))];
+    if (lane == 4) t = rhs;
+#pragma unroll
+    for (int q = 0; q < l; ++q) t = __fma_rn(-L[q], __shfl_sync(FULL, L[q], l), t);
+    const double pivot = __shfl_sync(FULL, t, l);
+    if (!(pivot > 0.0)) return -1;
+    diag[l] = __dsqrt_rn(pivot);
+    L[l] = __ddiv_rn(lane > l && lane <= 4 ? t : diag[l], diag[l]);
+    if (lane == l) L[l] = diag[l];
   }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 3; k >= 0; --k) {
+    double t = __shfl_sync(FULL, L[k], 4);
 #pragma unroll
-    for (int l = 0; l <= k; ++l) {
-      float t = (float)m[ix[k][l]] * sc[k] * sc[l];
-#pragma unroll
-      for (int q = 0; q < l; ++q) t = fmaf(-L[k][q], L[l][q], t);
-      if (k == l) {
-        ok = ok && t > 1e-3f;
-        inv[k] = ok ? rsqrtf(t) : 0.f;
-      } else {
-        L[k][l] = t * inv[l];
-      }
-    }
-  }
-  if (!ok) return chol_solve4(m, r, d);
-  double res[4] = {r[0], r[1], r[2], r[3]};
-#pragma unroll
-  for (int pass = 0; pass < 2; ++pass) {
-    float z[4];
-    double dd[4];
-    // scaled by a power of two near the residual's size: no FP32 underflow
-    const double big = fmax(fmax(fabs(res[0]), fabs(res[1])), fmax(fabs(res[2]), fabs(res[3])));
-    const long long eb = __double_as_longlong(big) & 0x7FF0000000000000ll;
-    if (eb < (64ll << 52) || eb > (1982ll << 52)) {
-      if (big == 0.0) {
-        if (pass == 0) d[0] = d[1] = d[2] = d[3] = 0.0;
-        break;
-      }
-      return chol_solve4(m, r, d);
-    }
-    const double up = __longlong_as_double((2046ll << 52) - eb), dn = __longlong_as_double(eb);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      float t = (float)(res[k] * up) * sc[k];
-#pragma unroll
-      for (int q = 0; q < k; ++q) t = fmaf(-L[k][q], z[q], t);
-      z[k] = t * inv[k];
-    }
-#pragma unroll
-    for (int k = 3; k >= 0; --k) {
-      float t = z[k];
-#pragma unroll
-      for (int q = k + 1; q < 4; ++q) t = fmaf(-L[q][k], z[q], t);
-      z[k] = t * inv[k];
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      dd[k] = (double)(z[k] * sc[k]) * dn;
-      d[k] = pass == 0 ? dd[k] : d[k] + dd[k];
-    }
-    if (pass == 0) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int l = 0; l < 4; ++l) res[k] = __fma_rn(-m[ix[k][l]], dd[l], res[k]);
-    }
+    for (int q = k + 1; q < 4; ++q) t = __fma_rn(-__shfl_sync(FULL, L[k], q), d[q], t);
+    d[k] = __ddiv_rn(t, diag[k]);
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k)
@@ -592,14 +590,50 @@ __device__ __forceinline__ int solve4(const double m[10], const double r[4], dou
   return 0;
 }
 
-enum { STEP = 0, CONVERGED = 1, GIVE_UP = 2 };
+// CONVERGED: and the moments within qoi_check; MOMENTS_OFF: converged, but not that
+enum { STEP = 0, CONVERGED = 1, MOMENTS_OFF = 2, GIVE_UP = 3 };
+
+// One turn of round1_warp on the sums, by the first warp of block SOLVER: the
+// verdict and the next multipliers to every block.
+__device__ __forceinline__ void decide(const ParamsK& pr, ClusterShared& sh, int it, int lane) {
+  const int k = lane & 3;
+  const double A = sh.tot[k], Q = sh.Q[k], gk = __dsub_rn(A, Q);
+  const double S = k == 1 ? sh.tot[S1] : A;
+  int verdict = STEP;
+  double next = 0.0;
+  if (!__all_sync(FULL, isfinite(gk) && isfinite(S))) {
+    verdict = GIVE_UP;
+  } else {
+    const double r = __ddiv_rn(fabs(gk), S > 0.0 ? S : 1e-300);
+    if (!__all_sync(FULL, isfinite(r))) {
+      verdict = GIVE_UP;
+    } else if (__all_sync(FULL, r <= pr.tol)) {
+      const double den = k == 1 ? sh.S1 : Q;
+      verdict = __all_sync(FULL, __ddiv_rn(fabs(gk), den > 0.0 ? den : 1e-300) <= pr.qoi_check)
+                    ? CONVERGED
+                    : MOMENTS_OFF;
+    } else if (it == pr.max_iter) {
+      verdict = GIVE_UP;
+    } else {
+      double d[4];
+      if (solve_rows(sh, gk, d, lane) != 0) verdict = GIVE_UP;
+      else
+        next = __fma_rn(pr.step_s, k == 0 ? d[0] : (k == 1 ? d[1] : (k == 2 ? d[2] : d[3])),
+                        sh.lam[k]);
+    }
+  }
+  __syncwarp();  // lam and tot have been read
+  if (verdict == STEP) put_f64(&sh.lam[k], lane >> 2, next);
+  if (lane < CL) put_u32(&sh.verdict, lane, (unsigned)verdict);
+}
 
 // One histogram by the cluster; false when it is left to the warp kernels.
-__device__ bool process_cluster(const FusedArgs& a, ClusterShared& sh, long long b, int& turn,
+__device__ bool process_cluster(const FusedArgs& a, ClusterShared& sh, long long b,
                                 unsigned rank) {
   const GridK& g = a.grid;
   const ParamsK& pr = a.prm;
   const int P = g.P, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cw = (int)rank * CWARPS + warp;  // the warp in the cluster
   const int p = (int)rank * CT + tid;
   const bool in = p < P;
   const int j = in ? p / g.n_par : 0, i = in ? p - j * g.n_par : 0;
@@ -617,33 +651,26 @@ __device__ bool process_cluster(const FusedArgs& a, ClusterShared& sh, long long
       const unsigned long long t = __shfl_xor_sync(FULL, um, o);
       um = t > um ? t : um;
     }
-    const int bd = __any_sync(FULL, !fine && u != 0x8000000000000000ull);
-    if (lane < CL) {
-      put_u64(&sh.umax[rank * CWARPS + warp], lane, um);
-      put_u32(&sh.bad[rank * CWARPS + warp], lane, (unsigned)bd);
-    }
+    // a value that is not valid shows as the largest pattern
+    if (__any_sync(FULL, !fine && u != 0x8000000000000000ull)) um = ~0ull;
+    if (lane < CL) put_u64(&sh.umax[cw], lane, um);
   }
   cluster_sync();
   unsigned long long us = 0;
-  int bad = 0;
-  for (int w = 0; w < CL * CWARPS; ++w) {
-    us = sh.umax[w] > us ? sh.umax[w] : us;
-    bad |= sh.bad[w];
-  }
-  if (bad || us == 0) return false;  // the same in every block
+  for (int w = 0; w < CL * CWARPS; ++w) us = sh.umax[w] > us ? sh.umax[w] : us;
+  if (us == ~0ull || us == 0) return false;  // the same in every block
   const double s = __longlong_as_double((long long)us), ebound = __dmul_rn(pr.tau, s);
-  double Q[4], S1;  // S_k = Q_k but for k = 1 (x >= 0)
-  {
-    const double w = vol * x, wv = w * v;
-    double t[CV] = {w, wv, w * v2, wv * v, fabs(wv)};
-    cluster_sums(sh, t, turn, rank);
-    __syncthreads();
-    for (int k = 0; k < 4; ++k) Q[k] = sh.tot[k];
-    S1 = sh.tot[4];
+  // Q_k and S_1 of x (x >= 0: S_k = Q_k for the others)
+  if (in) send_terms<false>(sh, p, __dmul_rn(vol, x), v, v2);
+  sum_terms(g, sh, rank, S1);
+  if (rank == SOLVER && warp == 0) {
+    if (lane < 4) sh.Q[lane] = sh.tot[lane];
+    if (lane == 4) sh.S1 = sh.tot[S1];
+    __syncwarp();
   }
   unsigned st = 0;
-  int total_it = 0, code = 0;
-  double xp = 0.0, f = 0.0, escapes = 0.0;
+  int total_it = 0, code = 0, escapes = 0, before = 0;
+  double xp = 0.0, f = 0.0;
   bool done = false;
   for (int level = 0; level < 2 && !done; ++level) {
     const double dl = bin_width(pr.tau, s, level ? pr.alpha4 : pr.alpha);
@@ -660,79 +687,56 @@ __device__ bool process_cluster(const FusedArgs& a, ClusterShared& sh, long long
         sh.tb[jt] = corr_b(lam, g.vperp2[jt]);
       __syncthreads();
       f = in ? corr_kl(xp, sh.ta[i], sh.tb[j]) : 0.0;
-      const double fv = f * vol, wv = fv * v, wvv = wv * v;
-      double t[CV] = {fv, wv, fv * v2, wvv, fabs(wv), wv * v2, wvv * v, fv * v2 * v2, wvv * v2,
-                      wvv * v * v, code == AEQC_CODE_ESCAPE ? 1.0 : 0.0, code != 0 ? 1.0 : 0.0,
-                      in && !(fabs(f - x) <= ebound) ? 1.0 : 0.0};
-      cluster_sums(sh, t, turn, rank);
-      if (warp == 0) {
-        double A[4], gk[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          A[k] = sh.tot[k];
-          gk[k] = A[k] - Q[k];
-        }
-        const double S[4] = {A[0], sh.tot[4], A[2], A[3]};
-        const double res = scaled_residual(gk, S);
-        int vd = STEP;
-        if (!isfinite(res)) vd = GIVE_UP;
-        else if (res <= pr.tol) vd = CONVERGED;
-        else if (it == pr.max_iter) vd = GIVE_UP;
-        else {
-          const double m[10] = {A[0], A[1], A[2], A[3], A[3],
-                                sh.tot[5], sh.tot[6], sh.tot[7], sh.tot[8], sh.tot[9]};
-          double d[4];
-          if (solve4(m, gk, d) != 0) vd = GIVE_UP;
-          else if (lane < 4)
-            sh.lam[lane] = lam[lane] + pr.step_s * (lane == 0 ? d[0] : lane == 1 ? d[1]
-                                                    : lane == 2 ? d[2] : d[3]);
-        }
-        if (lane == 0) sh.verdict = vd;
-      }
-      __syncthreads();
+      if (in) send_terms<true>(sh, p, __dmul_rn(f, vol), v, v2);
+      sum_terms(g, sh, rank, M33);
+      if (rank == SOLVER && warp == 0) decide(pr, sh, it, lane);
+      cluster_sync();
       verdict = sh.verdict;
-      if (verdict == CONVERGED) total_it += it;
+      if (verdict != STEP) total_it += it;
     }
-    if (verdict == GIVE_UP) return false;  // every block's totals are the same
-    escapes = sh.tot[10];
+    if (verdict == GIVE_UP) return false;
+    // end-to-end check: what each warp of the cluster found
+    const unsigned esc = __ballot_sync(FULL, in && code == AEQC_CODE_ESCAPE);
+    const int viol = __any_sync(FULL, in && !(fabs(f - x) <= ebound));
+    const int nonzero = __any_sync(FULL, in && code != 0);
+    if (lane < CL)
+      put_u32(&sh.flags[cw], lane,
+              (unsigned)__popc(esc) | (viol ? 256u : 0u) | (nonzero ? 512u : 0u));
+    cluster_sync();
+    const unsigned f0 = sh.flags[lane], f1 = lane + 32 < CL * CWARPS ? sh.flags[lane + 32] : 0u;
+    escapes = __reduce_add_sync(FULL, (int)(f0 & 255u) + (int)(f1 & 255u));
+    before = __reduce_add_sync(FULL, (lane < cw ? (int)(f0 & 255u) : 0) +
+                                         (lane + 32 < cw ? (int)(f1 & 255u) : 0));
     st = AEQC_ST_CONVERGED | (level ? AEQC_ST_ALPHA_RETRY : 0u) |
-         (escapes > 0.0 ? AEQC_ST_CODE_ESCAPE : 0u) | (sh.tot[11] > 0.0 ? 0u : AEQC_ST_AE_EXACT);
-    bool ok = sh.tot[12] == 0.0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const double den = k == 1 ? S1 : Q[k];
-      ok = ok && fabs(sh.tot[k] - Q[k]) / (den > 0.0 ? den : 1e-300) <= pr.qoi_check;
-    }
-    done = ok;
-    __syncthreads();  // tot and lam have been read by all before they change
+         (escapes > 0 ? AEQC_ST_CODE_ESCAPE : 0u) |
+         (__any_sync(FULL, (f0 | f1) & 512u) ? 0u : AEQC_ST_AE_EXACT);
+    done = verdict == CONVERGED && !__any_sync(FULL, (f0 | f1) & 256u);
   }
   if (!done) {
     st = AEQC_ST_VERBATIM | AEQC_ST_ALPHA_RETRY;
     code = AEQC_CODE_ESCAPE;
     f = x;
-    escapes = (double)P;
+    escapes = P;
+    before = (int)rank * CT + 32 * warp;
   }
   const long long o = b * (long long)P + p;
   if (in) a.codes[o] = (int16_t)code;
   if (in && a.f_out) a.f_out[o] = f;
-  if (a.out.count && escapes > 0.0) {
+  if (a.out.count && escapes > 0) {
     // positions in the outlier list: one range per histogram, in point order
     const unsigned m = __ballot_sync(FULL, in && code == AEQC_CODE_ESCAPE);
-    if (lane < CL) put_u32(&sh.esc[rank * CWARPS + warp], lane, (unsigned)__popc(m));
-    const long long cnt = (long long)escapes;
     if (rank == 0 && tid == 0) {
       const unsigned long long base =
-          atomicAdd((unsigned long long*)a.out.count, (unsigned long long)cnt);
+          atomicAdd((unsigned long long*)a.out.count, (unsigned long long)escapes);
       for (unsigned r = 0; r < CL; ++r) put_u64(&sh.base, r, base);
     }
     cluster_sync();
-    long long pos = sh.base + __popc(m & ((1u << lane) - 1u));
-    for (int w = 0; w < (int)rank * CWARPS + warp; ++w) pos += sh.esc[w];
+    const long long pos = sh.base + before + __popc(m & ((1u << lane) - 1u));
     if (in && code == AEQC_CODE_ESCAPE && pos < a.out.capacity) {
       a.out.index[pos] = (a.row0 + b) * (long long)P + p;
       a.out.value[pos] = x;
     }
-    if (sh.base + cnt > a.out.capacity) st |= AEQC_ST_OUTLIER_OVERFLOW;
+    if (sh.base + escapes > a.out.capacity) st |= AEQC_ST_OUTLIER_OVERFLOW;
   }
   if (rank == 0 && tid < 4) a.lambda[b * 4 + tid] = done ? sh.lam[tid] : 0.0;
   if (rank == 0 && tid == 0) {
@@ -757,12 +761,12 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(CT, 3)
   // to have started, which a barrier of the cluster shows and nothing else does
   // (process_cluster writes into all eight blocks before its first barrier).
   cluster_sync();
-  int turn = 0;
+  load_weights(a.grid, sh);
   const int nc = gridDim.x / CL;
   if (all && blockIdx.x == 0 && threadIdx.x == 0) *count = all;
   for (int t = blockIdx.x / CL; t < cnt; t += nc) {
     const int b = all ? t : list[t];
-    const bool done = process_cluster(a, sh, b, turn, rank);
+    const bool done = process_cluster(a, sh, b, rank);
     // the blocks leave the histogram together: nobody writes into the shared
     // memory of one that still reads, or has ended; and every block has read
     // the entry before it changes
@@ -1152,9 +1156,7 @@ unsigned cluster_grid(long long most) {
   return (unsigned)((c > 0 ? c : 1) * CL);
 }
 
-// Histograms up to which the clusters take a call or a list.  FP64 form of n
-// histograms, clusters / warps: n = 1 49 / 340 us, 16 59 / 364, 64 118 / 647,
-// 128 216 / 648, 256 422 / 649, 512 879 / 650 us.
+// Histograms up to which the clusters take a call or a list (times at the kernel).
 constexpr int CLUSTER_MOST = 320;
 
 }  // namespace
