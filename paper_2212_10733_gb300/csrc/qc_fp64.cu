@@ -1156,8 +1156,17 @@ unsigned cluster_grid(long long most) {
   return (unsigned)((c > 0 ? c : 1) * CL);
 }
 
-// Histograms up to which the clusters take a call or a list (times at the kernel).
-constexpr int CLUSTER_MOST = 320;
+// Histograms of P points up to which the clusters take a call or a list.  A
+// cluster's time hardly depends on P (57 of them run at once, about 1.1 us a
+// histogram at P = 100 and 1.5 at 1,521); a warp's does, 140 us at P = 100,
+// 185 at 225, 325 at 625 and 730 at 1,521, whatever the number.  Both take the
+// same time at 76 histograms for P = 49 and 64, 110 to 160 for P = 70 and 100,
+// about 180 for 225, 250 for 625, 470 for 1,521: the line runs below these.
+// Few points leave the system close to singular; what round 1 does not solve,
+// the clusters try in vain and the warps do again (P = 20: 57 histograms 653
+// instead of 411 us, P = 35: 76 603 instead of 460), so such grids go to the
+// warps at once.
+int cluster_most(int P) { return P < 64 ? 0 : (P < 992 ? 72 + P / 4 : 320); }
 
 }  // namespace
 
@@ -1166,9 +1175,10 @@ static int launch_fused_fp64_rest(const FusedArgs& a, const int* list, const int
 
 int launch_fused_fp64(const FusedArgs& a, cudaStream_t s) {
   if (a.n <= 0) return AEQC_OK;
-  if (a.n <= CLUSTER_MOST && cluster_form(a)) {
-    fused_fp64_cluster_kernel<<<cluster_grid(a.n), CT, 0, s>>>(a, a.fb_list, a.fb_count,
-                                                               CLUSTER_MOST, (int)a.n);
+  const int most = cluster_most(a.grid.P);
+  if (a.n <= most && cluster_form(a)) {
+    fused_fp64_cluster_kernel<<<cluster_grid(a.n), CT, 0, s>>>(a, a.fb_list, a.fb_count, most,
+                                                               (int)a.n);
     int rc = check_launch("fused_fp64_cluster_kernel");
     return rc ? rc : launch_fused_fp64_rest(a, a.fb_list, a.fb_count, s);
   }
@@ -1183,8 +1193,9 @@ int launch_fused_fp64(const FusedArgs& a, cudaStream_t s) {
 
 int launch_fused_fp64_list(const FusedArgs& a, int* list, int* count, cudaStream_t s) {
   if (a.n <= 0) return AEQC_OK;
-  if (cluster_form(a)) {
-    fused_fp64_cluster_kernel<<<cluster_grid(a.n), CT, 0, s>>>(a, list, count, CLUSTER_MOST, 0);
+  const int most = cluster_most(a.grid.P);
+  if (most > 0 && cluster_form(a)) {
+    fused_fp64_cluster_kernel<<<cluster_grid(a.n), CT, 0, s>>>(a, list, count, most, 0);
     int rc = check_launch("fused_fp64_cluster_kernel");
     if (rc) return rc;
   }

@@ -87,6 +87,22 @@ def test_fp64_form_of_a_few_and_of_many(aq, grid, tau, options, n):
     np.testing.assert_array_equal(bits(few.f), bits(many.f[:n]), err_msg="f")
 
 
+@pytest.mark.parametrize("grid,line", [((7, 9), 63), ((8, 8), 88), ((10, 10), 97),
+                                       ((39, 25), 315), ((31, 32), 320)])
+def test_fp64_form_on_both_sides_of_the_line(aq, grid, line):
+    """The number of histograms that clusters take depends on the points of one."""
+    g = aq.Grid(*synth.grid_arrays(*grid))
+    P = grid[0] * grid[1]
+    x, xh = batch(line + 1, grid, 1e-3, 17)
+    p = aq.params_default(tau=1e-3, kernel=aq.KERNEL_FP64)
+    a, b = (aq.quantize_correct(g, x[:n].contiguous(), xh[:n].contiguous(), p,
+                                outlier_capacity=n * P, want_f=True) for n in (line, line + 1))
+    torch.cuda.synchronize()
+    for name in FIELDS + ("f",):
+        np.testing.assert_array_equal(bits(getattr(a, name)), bits(getattr(b, name)[:line]),
+                                      err_msg=name)
+
+
 @pytest.mark.parametrize("grid", [(39, 39), (20, 20)])
 @pytest.mark.parametrize("tau", [1e-4, 1e-3])
 def test_fast_form_in_pieces(aq, grid, tau):
