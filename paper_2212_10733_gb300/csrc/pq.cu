@@ -210,23 +210,24 @@ __device__ __forceinline__ void for_elements(const void* z, int bf16, long long 
   for (; r < r1; r += step, e += estep) body(e, d, load_z(z, bf16, e));
 }
 
-// True in every thread of the last of the group's blocks to arrive; what the
-// others wrote before is then visible.  The counter is left at zero.
-__device__ __forceinline__ bool last_block_of_group(int* done) {
+// True in every thread of the last of the group's blocks to arrive at its
+// counter; what the others wrote before is then visible.  The counter is left at
+// zero.
+__device__ __forceinline__ bool last_block_of_group(int* counter) {
   __shared__ int last;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
-    last = atomicAdd(&done[blockIdx.y], 1) == (int)gridDim.x - 1;
-    if (last) done[blockIdx.y] = 0;
+    last = atomicAdd(counter, 1) == (int)gridDim.x - 1;
+    if (last) *counter = 0;
   }
   __syncthreads();
   if (last) __threadfence();
   return last;
 }
 
-__global__ void pq_clear_kernel(int* keys, long long* acc, unsigned long long* cnt, int* done,
-                                int G, int GL, int k) {
+__global__ void pq_clear_kernel(int* keys, long long* acc, unsigned long long* cnt, int GL,
+                                int k) {
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < GL * k; t += gridDim.x * blockDim.x) {
     acc[t] = 0;
     cnt[t] = 0;
@@ -234,16 +235,18 @@ __global__ void pq_clear_kernel(int* keys, long long* acc, unsigned long long* c
       keys[2 * t] = 0x7FFFFFFF;    // running minimum
       keys[2 * t + 1] = (int)0x80000000;  // running maximum
     }
-    if (t < G) done[t] = 0;
   }
 }
 
 // Range of each column; the group's last block then sets the start centroids
 // and the fixed-point scale of each dimension (one launch, and one thread per
-// centroid: as a kernel of its own with a thread per column it took 11 us).
+// centroid: as a kernel of its own with a thread per column it took 11 us).  The
+// group's counter is the low word of its first member count, zero until the
+// iterations; theirs is its first key, which is read here for the last time.
 __global__ void pq_minmax_init_kernel(const void* z, int bf16, long long n, int L,
-                                      const long long* off, int* keys, int* done, int k,
-                                      float* table, int* shift) {
+                                      const long long* off, int* keys,
+                                      unsigned long long* cnt, int k, float* table,
+                                      int* shift) {
   __shared__ int smin[PQ_THREADS], smax[PQ_THREADS];
   int mn = 0x7FFFFFFF, mx = (int)0x80000000;
   for_elements(z, bf16, n, L, off, [&](long long, int, float v) {
@@ -265,8 +268,8 @@ __global__ void pq_minmax_init_kernel(const void* z, int bf16, long long n, int 
     atomicMin(&keys[2 * gd], mn);
     atomicMax(&keys[2 * gd + 1], mx);
   }
-  if (!last_block_of_group(done)) return;
   const int g = blockIdx.y;
+  if (!last_block_of_group(reinterpret_cast<int*>(&cnt[(long long)g * L * k]))) return;
   const long long ng = group_hi(off, g, n) - group_lo(off, g, n);
   for (int t = threadIdx.x; t < L * k; t += blockDim.x) {
     const int gd = g * L + t / k, j = t % k;
@@ -277,6 +280,8 @@ __global__ void pq_minmax_init_kernel(const void* z, int bf16, long long n, int 
     table[(long long)g * L * k + t] = none ? 0.f : start_centroid(lo, hi, j, k);
     if (j == 0) shift[gd] = fixed_shift(lo, hi, ng);
   }
+  __syncthreads();
+  if (threadIdx.x == 0) keys[2 * g * L] = 0;
 }
 
 // One Lloyd iteration: every value is assigned to its nearest centroid and
@@ -290,7 +295,7 @@ __global__ void pq_minmax_init_kernel(const void* z, int bf16, long long n, int 
 template <int STEPS>
 __global__ void __launch_bounds__(PQ_THREADS) pq_accum_kernel(
     const void* z, int bf16, long long n, int L, const long long* off, int k, int k2,
-    float* table, const int* shift, long long* acc, unsigned long long* cnt, int* done) {
+    float* table, const int* shift, long long* acc, unsigned long long* cnt, int* keys) {
   extern __shared__ __align__(16) unsigned char sm[];
   float* c = reinterpret_cast<float*>(sm);                     // [k2][L]
   unsigned* slo = reinterpret_cast<unsigned*>(c + L * k2);     // [k][L]
@@ -322,7 +327,7 @@ __global__ void __launch_bounds__(PQ_THREADS) pq_accum_kernel(
       atomicAdd(&cnt[o], (unsigned long long)scnt[t]);
     }
   }
-  if (!last_block_of_group(done)) return;
+  if (!last_block_of_group(&keys[2 * g * L])) return;
   for (int t = threadIdx.x; t < L * k; t += blockDim.x) {
     const long long o = (long long)g * L * k + t;
     const unsigned long long ct = __ldcg(&cnt[o]);
@@ -659,17 +664,24 @@ size_t encode_smem(int L, int k2) { return 4 * (size_t)L * ((size_t)k2 + 1); }
 
 using namespace aeqc;
 
-extern "C" size_t pq_train_workspace_size(int32_t G, int32_t L, int32_t k) {
-  if (G < 1 || L < 1 || k < 2) return 0;
+static size_t counts_bytes(int32_t G, int32_t L) {
+  return use_counts(G, L) ? sizeof(unsigned) * (size_t)G * L * PQ_BINS : 0;
+}
+
+// what every call needs: the sums of the iterations
+static size_t sums_bytes(int32_t G, int32_t L, int32_t k) {
   WsSize w;
   const size_t GL = (size_t)G * L;
   w.add<int>(2 * GL);
   w.add<int>(GL);
   w.add<long long>(GL * k);
   w.add<unsigned long long>(GL * k);
-  w.add<int>(G);
-  if (use_counts(G, L)) w.add<unsigned>(GL * PQ_BINS);
   return w.bytes;
+}
+
+extern "C" size_t pq_train_workspace_size(int32_t G, int32_t L, int32_t k) {
+  if (G < 1 || L < 1 || k < 2) return 0;
+  return sums_bytes(G, L, k) + counts_bytes(G, L);
 }
 
 extern "C" int pq_train(const void* z, int32_t latent_dtype, int64_t n, int32_t L,
@@ -681,8 +693,7 @@ extern "C" int pq_train(const void* z, int32_t latent_dtype, int64_t n, int32_t 
   AEQC_CHECK_ARG(table && workspace && (z || n == 0), "pq_train: null pointer");
   AEQC_CHECK_ARG(G == 1 || group_offsets, "pq_train: G > 1 needs group_offsets");
   AEQC_CHECK_ARG(iters >= 0 && iters <= 10000, "pq_train: iters=%d", iters);
-  AEQC_CHECK_ARG(workspace_bytes >= pq_train_workspace_size(G, L, k),
-                 "pq_train: workspace too small");
+  AEQC_CHECK_ARG(workspace_bytes >= sums_bytes(G, L, k), "pq_train: workspace too small");
   AEQC_CHECK_ARG(accum_limit(L, k) <= 200 * 1024, "pq_train: L * k = %d too large", L * k);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -693,12 +704,13 @@ extern "C" int pq_train(const void* z, int32_t latent_dtype, int64_t n, int32_t 
   int* shift = c.take<int>(GL);
   long long* acc = c.take<long long>((size_t)GL * k);
   unsigned long long* cnt = c.take<unsigned long long>((size_t)GL * k);
-  int* done = c.take<int>(G);
-  unsigned* counts = use_counts(G, L) ? c.take<unsigned>((size_t)GL * PQ_BINS) : nullptr;
   AEQC_CHECK_ARG(c.ok(), "pq_train: workspace not 256-byte aligned");
+  // the counts where the workspace has room for them
+  const size_t cb = counts_bytes(G, L);
+  unsigned* counts = cb && c.left >= cb ? c.take<unsigned>((size_t)GL * PQ_BINS) : nullptr;
   const dim3 grid = pq_grid(G, n, L);
-  if (bf16 && use_counts(G, L) && n < (1ll << 32)) {
-    AEQC_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(unsigned) * (size_t)GL * PQ_BINS, s));
+  if (bf16 && counts && n < (1ll << 32)) {
+    AEQC_CUDA_TRY(cudaMemsetAsync(counts, 0, cb, s));
     const uint16_t* zb = static_cast<const uint16_t*>(z);
     // 16-byte loads: every row starts at a multiple of eight elements
     const bool vec = L % 8 == 0 && reinterpret_cast<uintptr_t>(z) % 16 == 0;
@@ -722,8 +734,8 @@ extern "C" int pq_train(const void* z, int32_t latent_dtype, int64_t n, int32_t 
     return check_launch("pq_lloyd_counts_kernel");
   }
   const int nb = (GL * k + 255) / 256;
-  pq_clear_kernel<<<nb, 256, 0, s>>>(keys, acc, cnt, done, G, GL, k);
-  pq_minmax_init_kernel<<<grid, PQ_THREADS, 0, s>>>(z, bf16, n, L, off, keys, done, k, table,
+  pq_clear_kernel<<<nb, 256, 0, s>>>(keys, acc, cnt, GL, k);
+  pq_minmax_init_kernel<<<grid, PQ_THREADS, 0, s>>>(z, bf16, n, L, off, keys, cnt, k, table,
                                                     shift);
   rc = check_launch("pq_minmax_init_kernel");
   if (rc) return rc;
@@ -735,7 +747,7 @@ extern "C" int pq_train(const void* z, int32_t latent_dtype, int64_t n, int32_t 
     const auto kernel = pq_accum_kernel<decltype(st)::value>;
     if (sm > 48 * 1024) rc = raise_smem_limit((const void*)kernel, (int)sm);
     for (int it = 0; it < iters && !rc; ++it)
-      kernel<<<grid, PQ_THREADS, sm, s>>>(z, bf16, n, L, off, k, k2, table, shift, acc, cnt, done);
+      kernel<<<grid, PQ_THREADS, sm, s>>>(z, bf16, n, L, off, k, k2, table, shift, acc, cnt, keys);
   });
   return rc ? rc : check_launch("pq_accum_kernel");
 }

@@ -226,3 +226,31 @@ def test_bf16_counts_equal_values(aq, n, L, G, k, kind):
     a = aq.pq_train(z, k=k, iters=6, group_offsets=goff, G=G)
     b = aq.pq_train(z.float(), k=k, iters=6, group_offsets=goff, G=G)
     np.testing.assert_array_equal(a.cpu().numpy().view(np.int32), b.cpu().numpy().view(np.int32))
+
+
+@pytest.mark.parametrize("dtype", ["bfloat16", "float32"])
+@pytest.mark.parametrize("n,L,G,k,iters", [(3000, 8, 1, 16, 4), (70000, 32, 2, 64, 2),
+                                           (500, 1, 3, 2, 3), (900, 16, 1, 256, 1)])
+def test_workspace_of_the_sums_alone(aq, n, L, G, k, iters, dtype):
+    """A workspace with room for the iterations' sums only (keys, shifts, sums and
+    member counts, each rounded to 256 bytes) is enough, with the same table; one
+    byte less is refused, and nothing behind the given bytes is touched."""
+    z = torch.as_tensor(latents(n, L, n), device=DEV).to(getattr(torch, dtype))
+    off = torch.as_tensor(np.linspace(0, n, G + 1).astype(np.int64), device=DEV)
+    goff = off if G > 1 else None
+    want = aq.pq_train(z, k=k, iters=iters, group_offsets=goff, G=G)
+    need = sum((b * G * L + 255) // 256 * 256 for b in (8, 4, 8 * k, 8 * k))
+    ws = torch.full((need + 65536,), 0x5A, dtype=torch.uint8, device=DEV)
+    got = torch.empty_like(want)
+
+    def call(nbytes):
+        aq._check(aq.load().pq_train(aq._ptr(z), aq._dtype_code(z.dtype), n, L, aq._ptr(goff), G,
+                                     k, iters, aq._ptr(got), aq._ptr(ws), nbytes, aq._stream()))
+
+    call(need)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(got.cpu().numpy().view(np.int32),
+                                  want.cpu().numpy().view(np.int32))
+    assert bool((ws[need:] == 0x5A).all())
+    with pytest.raises(aq.AeqcError):
+        call(need - 1)
