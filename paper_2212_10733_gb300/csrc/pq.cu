@@ -15,6 +15,7 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "aeqc_internal.cuh"
@@ -56,11 +57,27 @@ __device__ __forceinline__ long long group_hi(const long long* off, int g, long 
 // banks for L = 32), padded with +infinity to k2 rows (k2 >= k), and per
 // dimension lim: the distance up to which the bisection below may replace
 // the k distances.
+// The table goes through `stage` (L (k + 1) words) where there is one: written
+// straight to its place, a warp's 32 centroids of a dimension fall into one bank
+// (2,048 cycles of a block at L k = 2,048).
 __device__ __forceinline__ void load_table(const float* table, int L, int k, int k2, float* c,
-                                           int* lim) {
-  for (int t = threadIdx.x; t < L * k; t += blockDim.x) {
-    const int dd = t / k, j = t - dd * k;
-    c[j * L + dd] = table[t];
+                                           int* lim, float* stage = nullptr) {
+  if (stage) {
+    const int ks = k | 1;  // odd: the lanes of both copies in different banks
+    for (int t = threadIdx.x; t < L * k; t += blockDim.x) {
+      const int dd = t / k;
+      stage[dd * ks + (t - dd * k)] = table[t];
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < L * k; t += blockDim.x) {
+      const int j = t / L;
+      c[t] = stage[(t - j * L) * ks + j];
+    }
+  } else {
+    for (int t = threadIdx.x; t < L * k; t += blockDim.x) {
+      const int dd = t / k, j = t - dd * k;
+      c[j * L + dd] = table[t];
+    }
   }
   for (int t = L * k + threadIdx.x; t < L * k2; t += blockDim.x) c[t] = INFINITY;
   for (int t = threadIdx.x; t < L; t += blockDim.x) lim[t] = 0x7F000000;  // 2^127
@@ -289,9 +306,10 @@ __global__ void pq_minmax_init_kernel(const void* z, int bf16, long long n, int 
 // then one global add per cluster), and the group's last block moves the
 // centroids.  The totals are pairs of 32-bit words with the carry taken from
 // the value that the low word's add returns: 64-bit adds in shared memory are
-// compare-and-swap loops.  230 -> 138 us per iteration over 2^20 x 32 float32
-// latents with k = 16 (integer conversion, bisection, native adds, the move
-// of the centroids in the same launch), bound by instruction issue.
+// compare-and-swap loops.  Training on float32 latents of 32 dimensions, before
+// (64-bit adds, FP64 conversion, full search) and now: 10^6 rows, k = 16, four
+// iterations 957 and 500 us; 100,000 rows, ten iterations, k = 16 428 and 302, k =
+// 64 658 and 404 us; bound by instruction issue.
 template <int STEPS>
 __global__ void __launch_bounds__(PQ_THREADS) pq_accum_kernel(
     const void* z, int bf16, long long n, int L, const long long* off, int k, int k2,
@@ -303,8 +321,10 @@ __global__ void __launch_bounds__(PQ_THREADS) pq_accum_kernel(
   unsigned* scnt = shi + L * k;                                // [k][L]
   int* lim = reinterpret_cast<int*>(scnt + L * k);             // [L]
   const int g = blockIdx.y;
+  // (the sums' room, 3 L k words, for the table on its way in)
+  load_table(table + (long long)g * L * k, L, k, k2, c, lim, reinterpret_cast<float*>(slo));
   for (int t = threadIdx.x; t < L * k; t += blockDim.x) slo[t] = shi[t] = scnt[t] = 0u;
-  load_table(table + (long long)g * L * k, L, k, k2, c, lim);
+  __syncthreads();
   const int s = shift[g * L + threadIdx.x % L];
   const Range in = bisect_range(c + threadIdx.x % L, L, k, lim[threadIdx.x % L]);
   for_elements(z, bf16, n, L, off, [&](long long, int d, float v) {
@@ -318,23 +338,41 @@ __global__ void __launch_bounds__(PQ_THREADS) pq_accum_kernel(
     }
   });
   __syncthreads();
+  // global sums in the same order [k][L]: a warp's adds fall into whole lines
+  // (as [L][k], each lane's add was a transaction of its own)
+  const long long g0 = (long long)g * L * k;
   for (int t = threadIdx.x; t < L * k; t += blockDim.x) {
-    const int j = t / L, dd = t - j * L;
     if (scnt[t]) {
-      const long long o = (long long)g * L * k + dd * k + j;
-      atomicAdd(reinterpret_cast<unsigned long long*>(&acc[o]),
+      atomicAdd(reinterpret_cast<unsigned long long*>(&acc[g0 + t]),
                 (unsigned long long)shi[t] << 32 | slo[t]);
-      atomicAdd(&cnt[o], (unsigned long long)scnt[t]);
+      atomicAdd(&cnt[g0 + t], (unsigned long long)scnt[t]);
     }
   }
-  if (!last_block_of_group(&keys[2 * g * L])) return;
+  if (!keys || !last_block_of_group(&keys[2 * g * L])) return;
   for (int t = threadIdx.x; t < L * k; t += blockDim.x) {
-    const long long o = (long long)g * L * k + t;
-    const unsigned long long ct = __ldcg(&cnt[o]);
-    if (ct) table[o] = moved_centroid(__ldcg(&acc[o]), ct, shift[g * L + t / k]);
-    acc[o] = 0;
-    cnt[o] = 0;
+    const unsigned long long ct = __ldcg(&cnt[g0 + t]);
+    const int j = t / L, gd = g * L + t - j * L;
+    if (ct) table[(long long)gd * k + j] = moved_centroid(__ldcg(&acc[g0 + t]), ct, shift[gd]);
+    acc[g0 + t] = 0;
+    cnt[g0 + t] = 0;
   }
+}
+
+// The move of the centroids as a launch of its own, where a group has too many of
+// them for one block (the division is FP64 work: 10 us for 2,048).
+constexpr int PQ_MOVE_IN_BLOCK = 512;
+
+__global__ void pq_move_kernel(int G, int L, int k, const int* shift, long long* acc,
+                               unsigned long long* cnt, float* table) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (long long)G * L * k) return;
+  const unsigned long long ct = cnt[t];
+  const long long g = t / (L * k);
+  const int u = (int)(t - g * L * k), j = u / L;
+  const long long gd = g * L + u - j * L;
+  if (ct) table[gd * k + j] = moved_centroid(acc[t], ct, shift[gd]);
+  acc[t] = 0;
+  cnt[t] = 0;
 }
 
 // ---- Lloyd on value counts (bfloat16 latents) -----------------------------------
@@ -746,8 +784,17 @@ extern "C" int pq_train(const void* z, int32_t latent_dtype, int64_t n, int32_t 
   with_steps(steps, [&](auto st) {
     const auto kernel = pq_accum_kernel<decltype(st)::value>;
     if (sm > 48 * 1024) rc = raise_smem_limit((const void*)kernel, (int)sm);
-    for (int it = 0; it < iters && !rc; ++it)
-      kernel<<<grid, PQ_THREADS, sm, s>>>(z, bf16, n, L, off, k, k2, table, shift, acc, cnt, keys);
+    // rows of a block: at least twice as many as centroids to load and add up
+    const int64_t least = (pq_sms() + G - 1) / G, fit = n / (2 * (int64_t)G * k);
+    dim3 blocks = grid;
+    blocks.x = (unsigned)std::min<int64_t>(grid.x, std::max(least, fit));
+    const bool apart = L * k > PQ_MOVE_IN_BLOCK;
+    for (int it = 0; it < iters && !rc; ++it) {
+      kernel<<<blocks, PQ_THREADS, sm, s>>>(z, bf16, n, L, off, k, k2, table, shift, acc, cnt,
+                                          apart ? nullptr : keys);
+      if (apart)
+        pq_move_kernel<<<(GL * k + 127) / 128, 128, 0, s>>>(G, L, k, shift, acc, cnt, table);
+    }
   });
   return rc ? rc : check_launch("pq_accum_kernel");
 }
