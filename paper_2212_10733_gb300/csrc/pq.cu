@@ -623,12 +623,18 @@ size_t lloyd_smem(int k) { return 6 * (size_t)PQ_LCAP + 20 * (size_t)k; }
 // and 37 us without, at 2^20 rows 41 and 362 us.
 constexpr int64_t PQ_WINDOW_ROWS = 32768;
 
-// Counts are used for bfloat16 latents while the counts of all columns stay
+// Counts are possible for bfloat16 latents while the counts of all columns stay
 // within 16 MB (64 columns) and fit 32 bits.  Ten iterations over n x 32
 // latents, counted / one by one: n = 1,000 58 / 125 us, 10,000 68 / 214 us,
-// 100,000 93 / 592 us, 2^20 131 / 1,384 us; one iteration 30 / 23, 33 / 34,
-// 45 / 80, 73 / 190 us.
+// 100,000 93 / 302 us.
 bool use_counts(int G, int L) { return (long long)G * L <= 64; }
+
+// The counts cost a pass of their own, so the start table alone is made without
+// (100,000 x 7 latents, k = 16: 20 us, counted 50), and one iteration up to
+// 2^21 values (100,000 x 7 32 / 55 us; 100,000 x 32 59 / 53 us).
+bool counts_pay(int64_t n, int L, int iters) {
+  return iters >= 2 || (iters == 1 && n * L >= (1 << 21));
+}
 
 template <int STEPS>
 __global__ void __launch_bounds__(PQ_THREADS) pq_encode_kernel(
@@ -747,7 +753,7 @@ extern "C" int pq_train(const void* z, int32_t latent_dtype, int64_t n, int32_t 
   const size_t cb = counts_bytes(G, L);
   unsigned* counts = cb && c.left >= cb ? c.take<unsigned>((size_t)GL * PQ_BINS) : nullptr;
   const dim3 grid = pq_grid(G, n, L);
-  if (bf16 && counts && n < (1ll << 32)) {
+  if (bf16 && counts && n < (1ll << 32) && counts_pay(n, L, iters)) {
     AEQC_CUDA_TRY(cudaMemsetAsync(counts, 0, cb, s));
     const uint16_t* zb = static_cast<const uint16_t*>(z);
     // 16-byte loads: every row starts at a multiple of eight elements

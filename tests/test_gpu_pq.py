@@ -254,3 +254,14 @@ def test_workspace_of_the_sums_alone(aq, n, L, G, k, iters, dtype):
     assert bool((ws[need:] == 0x5A).all())
     with pytest.raises(aq.AeqcError):
         call(need - 1)
+
+
+@pytest.mark.parametrize("iters", [0, 1, 2])
+@pytest.mark.parametrize("n,L,k", [(1, 32, 16), (1000, 7, 64), (65535, 32, 16), (65536, 32, 16)])
+def test_few_iterations_counted_or_not(aq, n, L, k, iters):
+    """bfloat16 latents and the same values as float32 give the same table bit for
+    bit on both sides of the line from which they are counted."""
+    z = torch.as_tensor(latents(n, L, n + iters), device=DEV).to(torch.bfloat16)
+    a = aq.pq_train(z, k=k, iters=iters).cpu().numpy()
+    b = aq.pq_train(z.float(), k=k, iters=iters).cpu().numpy()
+    np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
