@@ -265,3 +265,14 @@ def test_few_iterations_counted_or_not(aq, n, L, k, iters):
     a = aq.pq_train(z, k=k, iters=iters).cpu().numpy()
     b = aq.pq_train(z.float(), k=k, iters=iters).cpu().numpy()
     np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
+
+
+@pytest.mark.parametrize("L,k", [(31, 66), (32, 64), (128, 16), (8, 256), (64, 64), (33, 62),
+                                 (64, 100)])
+def test_codes_with_tables_around_the_staged_sizes(aq, L, k):
+    """Tables of 2,046 entries, of 2,048 and of more, even and odd k, up to one that
+    has no room for the additional copy: the oracle's codes."""
+    z = latents(700, L, k)
+    t = np.ascontiguousarray(opq.init_centroids(z, k))
+    codes, _ = aq.pq_encode(torch.as_tensor(z, device=DEV), torch.as_tensor(t[None], device=DEV))
+    np.testing.assert_array_equal(codes.cpu().numpy(), opq.assign(z, t))
