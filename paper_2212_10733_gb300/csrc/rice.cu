@@ -604,6 +604,8 @@ __global__ void __launch_bounds__(128, 8) rice_unpack_kernel(const uint32_t* wor
     }
     __syncwarp();
   }
+  // the words asked for and not needed any more
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 }  // namespace
