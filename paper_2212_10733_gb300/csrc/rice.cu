@@ -87,18 +87,19 @@ __device__ __forceinline__ RowWords row_words(const int16_t* codes, long long b,
   return r;
 }
 
-// word lane + 32 i into w[i] (zero-level codes past the row), every load in
-// flight at once
+// word lane + 32 i into w[i] (zero-level codes past the row; NW words a lane hold
+// the row), every load in flight at once
+template <int NW>
 __device__ __forceinline__ void load_words(const RowWords& r, int P, int lane,
-                                           unsigned (&w)[RNW]) {
+                                           unsigned (&w)[NW]) {
   const unsigned* base = reinterpret_cast<const unsigned*>(r.row - r.par) + lane;
   if (!r.edge) {
 #pragma unroll
-    for (int i = 0; i < RNW; ++i)
+    for (int i = 0; i < NW; ++i)
       w[i] = lane + 32 * i < r.words ? __ldg(base + 32 * i) : 0x80018001u;
   } else {
 #pragma unroll
-    for (int i = 0; i < RNW; ++i) {
+    for (int i = 0; i < NW; ++i) {
       const int p = 2 * (lane + 32 * i) - r.par;
       const unsigned lo = p >= 0 && p < P ? (uint16_t)__ldg(r.row + p) : 0x8001u;
       const unsigned hi = p + 1 < P ? (uint16_t)__ldg(r.row + p + 1) : 0x8001u;
@@ -138,7 +139,12 @@ __device__ __forceinline__ int halves(unsigned v) { return (int)(v & 0xFFFFu) + 
 //    lo N for every j < lo with N the number of symbols below 2^(lo-1).
 // A tie goes to the smaller k.  Residual codes take four or five sums of the
 // sixteen, two symbols an instruction: 811 -> 300 us for 131,072 rows
-// of 1,521 codes.
+// of 1,521 codes.  NW words a lane hold a row: rows of up to RSMALL codes take the
+// form with four of them instead of twenty-five (20,000 rows of 10, measured and
+// packed: 103 -> 95 us).
+constexpr int RSMALL = 4 * 64 - 2;  // the row's words with one half at either end
+
+template <int NW>
 __global__ void __launch_bounds__(RW * 32) rice_measure_kernel(const int16_t* codes, long long n,
                                                                int P, uint8_t* kparam,
                                                                uint32_t* nbits,
@@ -148,16 +154,16 @@ __global__ void __launch_bounds__(RW * 32) rice_measure_kernel(const int16_t* co
   long long b = (long long)blockIdx.x * RW + (threadIdx.x >> 5);
   if (b >= n) return;
   RowWords r = row_words(codes, b, n, P);
-  unsigned ahead[RNW];  // the next row, loaded while this one is summed
+  unsigned ahead[NW];  // the next row, loaded while this one is summed
   load_words(r, P, lane, ahead);
   for (; b < n; b += nw) {
-    unsigned s[RNW], sum = 0, mx = 0;
+    unsigned s[NW], sum = 0, mx = 0;
     const int words = r.words;
     // the half past an odd end becomes the zero level: symbol 0 adds no prefix
     const int odd = (r.par + P) & 1 ? words - 1 - lane : -1;
     if (lane == 0 && r.par) ahead[0] = (ahead[0] & 0xFFFF0000u) | 0x8001u;
 #pragma unroll
-    for (int i = 0; i < RNW; ++i) {
+    for (int i = 0; i < NW; ++i) {
       if (32 * i >= words) break;
       if (32 * i == odd) ahead[i] = (ahead[i] & 0xFFFFu) | 0x80010000u;
       const unsigned v = symbols_of(ahead[i]);
@@ -178,7 +184,7 @@ __global__ void __launch_bounds__(RW * 32) rice_measure_kernel(const int16_t* co
       unsigned acc = 0, cap = 0;
       if (smax >= ((unsigned)RCAP << k)) {
 #pragma unroll
-        for (int i = 0; i < RNW; ++i) {
+        for (int i = 0; i < NW; ++i) {
           if (32 * i >= words) break;
           const unsigned t = prefixes(s[i], k);
           acc += t;
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(RW * 32) rice_measure_kernel(const int16_t* co
         }
       } else {
 #pragma unroll
-        for (int i = 0; i < RNW; ++i) {
+        for (int i = 0; i < NW; ++i) {
           if (32 * i >= words) break;
           acc += prefixes(s[i], k);
         }
@@ -206,7 +212,7 @@ __global__ void __launch_bounds__(RW * 32) rice_measure_kernel(const int16_t* co
       if (lo == 0) break;
       unsigned ge = 0;
 #pragma unroll
-      for (int i = 0; i < RNW; ++i) {
+      for (int i = 0; i < NW; ++i) {
         if (32 * i >= words) break;
         ge += min_u16x2((s[i] >> (lo - 1)) & ((0xFFFFu >> (lo - 1)) * 0x00010001u), 0x00010001u);
       }
@@ -646,7 +652,8 @@ extern "C" int rice_measure(const int16_t* codes, int64_t n, int32_t P, uint8_t*
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   long long blocks = (n + RW - 1) / RW;
   if (blocks > (long long)sms * 16) blocks = (long long)sms * 16;
-  rice_measure_kernel<<<(unsigned)blocks, RW * 32, 0, s>>>(codes, n, P, kparam, nbits, wc);
+  const auto measure = P <= RSMALL ? rice_measure_kernel<4> : rice_measure_kernel<RNW>;
+  measure<<<(unsigned)blocks, RW * 32, 0, s>>>(codes, n, P, kparam, nbits, wc);
   scan_block_sums<<<(unsigned)nb, 256, 0, s>>>(wc, n, bsum);
   scan_sums<<<1, SCAN_B, 0, s>>>(bsum, nb);
   scan_apply<<<(unsigned)nb, SCAN_B, 0, s>>>(wc, n, bsum, off);

@@ -127,3 +127,20 @@ def test_streams_any_alignment(aq, P, n, shift):
     np.testing.assert_array_equal(rs.offsets.cpu().numpy(), off)
     np.testing.assert_array_equal(rs.words.cpu().numpy().view(np.uint32), words)
     np.testing.assert_array_equal(aq.rice_decode(rs, P).cpu().numpy(), q)
+
+
+@pytest.mark.parametrize("P", [1, 2, 63, 253, 254, 255, 256])
+@pytest.mark.parametrize("n,shift", [(1, 1), (9, 0), (50, 1)])
+def test_streams_of_short_rows(aq, P, n, shift):
+    """Rows of one code to those around the longest that four words a lane hold, on
+    even and odd 2-byte boundaries."""
+    q = np.concatenate([mixed_codes(max(n, 4), P, 7 * P + n)])[:n]
+    flat = torch.full((n * P + 2,), 12345, dtype=torch.int16, device=DEV)
+    flat[shift:shift + n * P] = torch.as_tensor(q.reshape(-1), device=DEV)
+    rs = aq.rice_encode(flat[shift:shift + n * P].view(n, P))
+    ks, nb, off, words = orice.encode(q)
+    np.testing.assert_array_equal(rs.kparam.cpu().numpy(), ks)
+    np.testing.assert_array_equal(rs.nbits.cpu().numpy().astype(np.uint32), nb)
+    np.testing.assert_array_equal(rs.offsets.cpu().numpy(), off)
+    np.testing.assert_array_equal(rs.words.cpu().numpy().view(np.uint32), words)
+    np.testing.assert_array_equal(aq.rice_decode(rs, P).cpu().numpy(), q)
