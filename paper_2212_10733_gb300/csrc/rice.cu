@@ -11,12 +11,15 @@
 // at word offsets given by an exclusive prefix sum.
 //
 // rice_measure: warp per histogram, the symbols in registers, two to a word;
-// only the candidates that can still be the shortest are summed.  rice_pack: warp per histogram, each 32-symbol step
-// places its bit patterns with a warp prefix sum of their lengths and ORs
-// them into the histogram's stream in shared memory, which is then copied
-// out.  rice_unpack: one thread per histogram reads its stream through a
-// 64-bit bit buffer (reads never leave the histogram's words) and the warp
-// writes the decoded codes through shared memory in contiguous rows.
+// only the candidates that can still be the shortest are summed.
+// rice_pack: warp per histogram.  Rows of 993 codes and more (rice_pack_seg):
+// every lane appends the patterns of a run of consecutive symbols, placed by one
+// prefix sum of the runs' lengths.  Shorter rows (rice_pack): each 32-symbol step
+// places its patterns with a prefix sum of their lengths and ORs them into the
+// histogram's stream in shared memory.  Both copy the stream out from there.
+// rice_unpack: one thread per histogram reads its stream through a 64-bit buffer
+// filled from words copied ahead (reads never leave the histogram's words) and
+// the warp writes the decoded codes through shared memory in contiguous rows.
 #include "aeqc_internal.cuh"
 #include "workspace.cuh"
 
@@ -39,11 +42,6 @@ __device__ __forceinline__ int rice_code(unsigned s) {
   const unsigned z = s - 1u;
   const int q = (int)(z >> 1) ^ -(int)(z & 1u);
   return s == 0u ? AEQC_CODE_ZERO : (s == 65535u ? AEQC_CODE_ESCAPE : q);
-}
-
-__device__ __forceinline__ int rice_bits(unsigned s, int k) {
-  const unsigned u = s >> k;
-  return u < (unsigned)RCAP ? (int)u + 1 + k : RCAP + 16;
 }
 
 // ---- two symbols per 32-bit word --------------------------------------------------
