@@ -451,7 +451,14 @@ __global__ void __launch_bounds__(256) bias_act_tiny_kernel(const GemmArgs a) {
   }
 }
 
-constexpr long long SMALL_MAX_TILES = 76;
+// 128 x 128 tiles up to which the small form takes a product: half as many as SMs
+// with an FP64 A, three eighths with an FP32 one.
+long long small_tiles(bool a_f64) {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return (long long)sms * (a_f64 ? 4 : 3) / 8;
+}
 
 int launch_gemm(const GemmArgs& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0) return AEQC_OK;
@@ -476,11 +483,13 @@ int launch_gemm(const GemmArgs& a, cudaStream_t s) {
   if (tiles > 2147483647LL || tiles > 65535LL * 65535LL)
     return set_error(AEQC_EUNSUPPORTED, "gemm: too many row tiles");
   dim3 grid((a.N + BN - 1) / BN, (unsigned)tiles);
-  // up to half the SMs' worth of 128 x 128 tiles: 32 times as many small ones (a
-  // tile of the large form then waits alone on its SM for every load).  Encoding
-  // with H = 128: 10 rows 344 -> 69 us, 1,000 rows (8 tiles) 379 -> 87, 9,000
-  // rows (71 tiles) 454 -> 380 us.
-  if (a.n_groups <= 1 && tiles * grid.x <= SMALL_MAX_TILES) {
+  // few 128 x 128 tiles: 32 times as many small ones (a tile of the large form then
+  // waits alone on its SM for every load, 191 steps at K = 1521, and twice as long
+  // for FP64).  Encoding (FP64) with H = 128: 10 rows 344 -> 69 us, 1,000 rows (8
+  // tiles) 379 -> 87, 9,000 rows (71 tiles) 454 -> 380 us.  Decoding (FP32) with H =
+  // 512: 10 rows 100 -> 36 us, 500 rows (48 tiles) 118 -> 108, 700 rows (72 tiles)
+  // 118 -> 131 us.
+  if (a.n_groups <= 1 && tiles * grid.x <= small_tiles(a.a_f64)) {
     dim3 gs((a.N + SN_ - 1) / SN_, (unsigned)((a.M + SM_ - 1) / SM_));
     if (a.a_f64) gemm_small_kernel<true><<<gs, 256, 0, s>>>(a);
     else gemm_small_kernel<false><<<gs, 256, 0, s>>>(a);

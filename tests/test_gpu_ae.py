@@ -396,3 +396,18 @@ def test_small_batches_take_the_same_sums(aq, n, H, L):
     torch.cuda.synchronize()
     for a, b in ((z1, z2), (s1, s2), (h1, h2)):
         np.testing.assert_array_equal(a.cpu().numpy(), b[:n].cpu().numpy())
+
+
+@pytest.mark.parametrize("n", [512, 513, 640, 641, 768, 769])
+def test_decoded_rows_on_both_sides_of_the_small_form(aq, n):
+    """FP32 products of few rows (48, 60, 72 and 84 tiles of 128 x 128) take another
+    form than those of many and give the same bits."""
+    P, H, L = 1521, 512, 32
+    m = aq.Model(P, H, L)
+    m.set_group(0, synth.ae_init(P, H, L, 4))
+    z = torch.as_tensor(np.random.default_rng(n).standard_normal((2000, L)).astype(np.float32),
+                        device=DEV)
+    s = torch.linspace(0.5, 2.0, 2000, dtype=torch.float64, device=DEV)
+    many = aq.ae_decode(m, z, s)[:n, :P]
+    few = aq.ae_decode(m, z[:n].contiguous(), s[:n].contiguous())[:, :P]
+    assert torch.equal(few.contiguous().view(torch.int32), many.contiguous().view(torch.int32))
