@@ -402,7 +402,12 @@ size_t compress_batch_host_workspace_size(const aeqc_model* m, int64_t chunk,
 
 /* Decompression (end of Stage 5): decode the latents, x' from the codes,
  * f = x' exp(-lambda.phi) at every point (raw values at escapes, also
- * corrected), f [n][P] float64. */
+ * corrected), f [n][P] float64.  These are the values that compression with the
+ * same build checked, bit for bit.  The two exponentials a value is the product of
+ * are this library's own, within 0.503 units in the last place for arguments below
+ * 2^-4 and CUDA's exp beyond; a batch written by a build with another exponential
+ * (CUDA's throughout, before) is read back within three units in the last place
+ * of the values that build checked. */
 int decompress_batch(aeqc_model* m, const aeqc_grid* grid, const aeqc_compressed* in,
                      int64_t n, const int64_t* group_offsets, const aeqc_params* params,
                      double* f, void* workspace, size_t workspace_bytes, void* stream);

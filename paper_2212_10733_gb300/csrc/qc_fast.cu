@@ -361,11 +361,6 @@ struct Moments {
   unsigned flags;  // CODE_ESCAPE / AE_EXACT
 };
 
-// Sums over the warp of 32 64-bit values held by every lane, scattered:
-// lane k returns the total of value k.  Recursive halving: at each step a
-// lane keeps the half of its values selected by its lane bit and adds its
-// partner's copy of that half (the totals are bounded on the host so that
-// they fit).
 // Warp sums of four double-float values held by every lane: the total of
 // value k ends in lanes 8k..8k+7 (halving over lane bits 4 and 3, then a
 // butterfly over the remaining three bits), added error-free.
@@ -387,6 +382,11 @@ __device__ __forceinline__ df df_reduce_scatter4(const df (&a)[4], int lane) {
   return x;
 }
 
+// Sums over the warp of 32 64-bit values held by every lane, scattered:
+// lane k returns the total of value k.  Recursive halving: at each step a
+// lane keeps the half of its values selected by its lane bit and adds its
+// partner's copy of that half (the totals are bounded on the host so that
+// they fit).
 __device__ __forceinline__ long long reduce_scatter32(long long (&v)[32], int lane) {
 #pragma unroll
   for (int o = 16, n = 16; o >= 1; o >>= 1, n >>= 1) {
@@ -1679,8 +1679,7 @@ int make_fast_grid(const GridK& g, FastGridK* out) {
   memset(&f, 0, sizeof(f));
   *out = f;
   if (g.has_vol || g.n_par < 2 || g.n_perp < 2) return AEQC_OK;
-  // integer weights must stay below 2^24 (|i - i_c|^4, j^4) and the x' sums
-  // of one lane below 2^62
+  // integer weights must stay below 2^24 (|i - i_c|^4, j^4)
   if (g.n_par > 64 || g.n_perp > 64) return AEQC_OK;
   const double b = (g.vpar[g.n_par - 1] - g.vpar[0]) / (double)(g.n_par - 1);
   if (!(b > 0.0)) return AEQC_OK;
@@ -1699,9 +1698,9 @@ int make_fast_grid(const GridK& g, FastGridK* out) {
     if (fabs(g.vperp2[j] - d2 * (double)j * (double)j) > 1e-13 * g.vperp2[g.n_perp - 1])
       return AEQC_OK;
   // exact 64-bit moment sums: for every weight (i - i_c)^r j^(2q) of the
-  // moments, the sum of |weight| over the grid stays below 2^31, so that the
-  // totals of X' (split at bit 31: parts below 2^31 and 2^29) stay below 2^62;
-  // the residual rho (|rho| <= 2^37) enters only with the weights 1, i - i_c,
+  // moments, the sum of |weight| over the grid stays below 2^31 (strictly), so
+  // that the totals of X' (split at bit 32: parts below 2^32 and 2^28) stay below
+  // 2^63, the sign's bit; the residual rho (|rho| <= 2^37) enters only with the weights 1, i - i_c,
   // (i - i_c)^2 and j^2, whose sums must stay below 2^25
   {
     double wsum[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
