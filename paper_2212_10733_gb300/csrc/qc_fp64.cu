@@ -1156,17 +1156,27 @@ unsigned cluster_grid(long long most) {
   return (unsigned)((c > 0 ? c : 1) * CL);
 }
 
-// Histograms of P points up to which the clusters take a call or a list.  A
-// cluster's time hardly depends on P (57 of them run at once, about 1.1 us a
-// histogram at P = 100 and 1.5 at 1,521); a warp's does, 140 us at P = 100,
-// 185 at 225, 325 at 625 and 730 at 1,521, whatever the number.  Both take the
-// same time at 76 histograms for P = 49 and 64, 110 to 160 for P = 70 and 100,
-// about 180 for 225, 250 for 625, 470 for 1,521: the line runs below these.
+// Histograms of P points up to which the clusters take a call or a list for which
+// there are as many warps as `warps`.  A cluster's time hardly depends on P (57 of
+// them run at once, 1.1 to 2 us a histogram with the steps it takes); a warp's
+// does, 100 to 140 us at P = 100, 165 to 270 at 400, 455 to 730 at 1,521, and is
+// the call's time while there is a warp for each.  Over bounds from 1e-4 to 0.1
+// the clusters were never slower up to 48 histograms at P = 64, 64 at 100, 96 at
+// 225 and 400, 128 at 625, 160 at 900 and 200 at 1,221 and 1,521 (320 at 1,521:
+// between 0.68 and 1.35 times a warp's time): the line runs below these.  A list
+// in a small batch has few warps, whose work the clusters do faster at any number.
 // Few points leave the system close to singular; what round 1 does not solve,
 // the clusters try in vain and the warps do again (P = 20: 57 histograms 653
-// instead of 411 us, P = 35: 76 603 instead of 460), so such grids go to the
-// warps at once.
-int cluster_most(int P) { return P < 64 ? 0 : (P < 992 ? 72 + P / 4 : 320); }
+// instead of 411 us), so such grids go to the warps at once.
+int cluster_most(int P, long long warps) {
+  if (P < 64) return 0;
+  const int line = 40 + P / 9;
+  return warps < line ? 320 : line;
+}
+
+// the list kernel's blocks: sized for a few percent of the batch; the grid-stride
+// loop covers any count
+int list_blocks(long long n) { return grid_for(n / 16 + 1, 2); }
 
 }  // namespace
 
@@ -1175,7 +1185,7 @@ static int launch_fused_fp64_rest(const FusedArgs& a, const int* list, const int
 
 int launch_fused_fp64(const FusedArgs& a, cudaStream_t s) {
   if (a.n <= 0) return AEQC_OK;
-  const int most = cluster_most(a.grid.P);
+  const int most = cluster_most(a.grid.P, a.n);
   if (a.n <= most && cluster_form(a)) {
     fused_fp64_cluster_kernel<<<cluster_grid(a.n), CT, 0, s>>>(a, a.fb_list, a.fb_count, most,
                                                                (int)a.n);
@@ -1193,7 +1203,7 @@ int launch_fused_fp64(const FusedArgs& a, cudaStream_t s) {
 
 int launch_fused_fp64_list(const FusedArgs& a, int* list, int* count, cudaStream_t s) {
   if (a.n <= 0) return AEQC_OK;
-  const int most = cluster_most(a.grid.P);
+  const int most = cluster_most(a.grid.P, (long long)WPC * list_blocks(a.n));
   if (most > 0 && cluster_form(a)) {
     fused_fp64_cluster_kernel<<<cluster_grid(a.n), CT, 0, s>>>(a, list, count, most, 0);
     int rc = check_launch("fused_fp64_cluster_kernel");
@@ -1209,9 +1219,7 @@ static int launch_fused_fp64_rest(const FusedArgs& a, const int* list, const int
     const int rc_attr = raise_smem_limit((const void*)fused_fp64_list_kernel, (int)smem);
     if (rc_attr) return rc_attr;
   }
-  // sized for a few percent of the batch; the grid-stride loop covers any count
-  long long warps = a.n / 16 + 1;
-  fused_fp64_list_kernel<<<grid_for(warps, 2), WPC * 32, smem, s>>>(a, list, count);
+  fused_fp64_list_kernel<<<list_blocks(a.n), WPC * 32, smem, s>>>(a, list, count);
   return check_launch("fused_fp64_list_kernel");
 }
 

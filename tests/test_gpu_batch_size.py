@@ -87,8 +87,8 @@ def test_fp64_form_of_a_few_and_of_many(aq, grid, tau, options, n):
     np.testing.assert_array_equal(bits(few.f), bits(many.f[:n]), err_msg="f")
 
 
-@pytest.mark.parametrize("grid,line", [((7, 9), 63), ((8, 8), 88), ((10, 10), 97),
-                                       ((39, 25), 315), ((31, 32), 320)])
+@pytest.mark.parametrize("grid,line", [((7, 9), 63), ((8, 8), 47), ((10, 10), 51),
+                                       ((39, 25), 148), ((39, 39), 209)])
 def test_fp64_form_on_both_sides_of_the_line(aq, grid, line):
     """The number of histograms that clusters take depends on the points of one."""
     g = aq.Grid(*synth.grid_arrays(*grid))
@@ -104,11 +104,10 @@ def test_fp64_form_on_both_sides_of_the_line(aq, grid, line):
 
 
 @pytest.mark.parametrize("grid", [(39, 39), (20, 20)])
-@pytest.mark.parametrize("tau", [1e-4, 1e-3])
-def test_fast_form_in_pieces(aq, grid, tau):
+@pytest.mark.parametrize("tau,n,piece", [(1e-4, 5000, 1250), (1e-3, 5000, 1250), (1e-2, 900, 300)])
+def test_fast_form_in_pieces(aq, grid, tau, n, piece):
     """The fast kernel's deferred list is above the limit in one call and below
-    it in the pieces (at the larger bound)."""
-    n, piece = 5000, 1250
+    it in the pieces (at the larger bounds)."""
     g = aq.Grid(*synth.grid_arrays(*grid))
     x, xh = batch(n, grid, tau, 5)
     p = aq.params_default(tau=tau, kernel=aq.KERNEL_FAST)
