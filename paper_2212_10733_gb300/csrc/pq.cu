@@ -359,7 +359,8 @@ __global__ void __launch_bounds__(PQ_THREADS) pq_accum_kernel(
 }
 
 // The move of the centroids as a launch of its own, where a group has too many of
-// them for one block (the division is FP64 work: 10 us for 2,048).
+// them for one block (the division is FP64 work): 64 x 16 centroids in the block,
+// 104 -> 112 us for four iterations over 10,000 rows and 138 -> 163 over 30,000.
 constexpr int PQ_MOVE_IN_BLOCK = 512;
 
 __global__ void pq_move_kernel(int G, int L, int k, const int* shift, long long* acc,

@@ -1159,7 +1159,7 @@ unsigned cluster_grid(long long most) {
 // Histograms of P points up to which the clusters take a call or a list for which
 // there are as many warps as `warps`.  A cluster's time hardly depends on P (57 of
 // them run at once, 1.1 to 2 us a histogram with the steps it takes); a warp's
-// does, 100 to 140 us at P = 100, 165 to 270 at 400, 455 to 730 at 1,521, and is
+// does, 104 to 158 us at P = 100, 172 to 270 at 400, 453 to 731 at 1,521, and is
 // the call's time while there is a warp for each.  Over bounds from 1e-4 to 0.1
 // the clusters were never slower up to 48 histograms at P = 64, 64 at 100, 96 at
 // 225 and 400, 128 at 625, 160 at 900 and 200 at 1,221 and 1,521 (320 at 1,521:
